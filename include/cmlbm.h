@@ -118,7 +118,9 @@ typedef struct cmlbm cmlbm_t;
  *                         GB300), or CMLBM_KERNEL_TMA (rows staged in shared memory by TMA).
  *                         PAIR covers D3Q27 with FP32 / BF16 / FP16 storage, periodic x and nx a
  *                         multiple of 64, in every collision form (PAIR_TWO_STEPS: the Maxwellian
- *                         attractor and standard compressibility only);
+ *                         attractor and standard compressibility only); AUTO also updates two
+ *                         cells per thread on D3Q27 grids of any other nx >= 8 and with x walls
+ *                         where a plane nx * ny holds at least 2048 cells;
  *                         TMA covers D3Q27 with FP32 / BF16 / FP16 storage, nx a multiple of 128,
  *                         the Maxwellian attractor, standard compressibility, and no slab. An
  *                         explicit choice the configuration cannot use fails with
@@ -334,7 +336,9 @@ CMLBM_API int cmlbm_halo_unpack(cmlbm_t* h, int face, const void* in, int where)
 CMLBM_API long long cmlbm_launch_count(const cmlbm_t* h);
 
 /* The step kernel the handle runs: CMLBM_KERNEL_DIRECT, CMLBM_KERNEL_PAIR,
- * CMLBM_KERNEL_PAIR_TWO_STEPS or CMLBM_KERNEL_TMA (what CMLBM_KERNEL_AUTO resolved to);
+ * CMLBM_KERNEL_PAIR_TWO_STEPS or CMLBM_KERNEL_TMA (what CMLBM_KERNEL_AUTO resolved to, as a
+ * value that an explicit request of the same configuration accepts: on grids that PAIR does not
+ * cover, AUTO answers CMLBM_KERNEL_DIRECT whichever of the two it runs there);
  * CMLBM_ERR_INVALID for a NULL handle. */
 CMLBM_API int cmlbm_step_kernel(const cmlbm_t* h);
 

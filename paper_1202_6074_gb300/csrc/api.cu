@@ -411,6 +411,7 @@ int cmlbm_create(const cmlbm_config* cfg, cmlbm_t** out) {
     }
     if (cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess) h->nsm = 1;
     if ((c.kernel == CMLBM_KERNEL_AUTO || big) && cm::pair_eligible(p, h->D, c.storage != CMLBM_F64)) p.pair = 1;
+    else if (c.kernel == CMLBM_KERNEL_AUTO && cm::ragged_pair_eligible(p, h->D, c.storage != CMLBM_F64)) p.pair = 2;
     const bool two_ok = cm::two_steps_eligible(p, h->D, c.storage == CMLBM_F32, slab);
     if (c.kernel == CMLBM_KERNEL_PAIR_TWO_STEPS && !two_ok) {
         cmlbm_destroy(h);
@@ -507,7 +508,7 @@ int cmlbm_step_kernel(const cmlbm_t* h) {
     if (!h) return CMLBM_ERR_INVALID;
     if (h->tma) return CMLBM_KERNEL_TMA;
     if (h->two_steps) return CMLBM_KERNEL_PAIR_TWO_STEPS;
-    return h->p.pair ? CMLBM_KERNEL_PAIR : CMLBM_KERNEL_DIRECT;
+    return h->p.pair == 1 ? CMLBM_KERNEL_PAIR : CMLBM_KERNEL_DIRECT;
 }
 
 size_t cmlbm_state_bytes(const cmlbm_t* h) { return h ? (size_t)h->Q * (size_t)h->p.S * h->esize : 0; }

@@ -43,7 +43,8 @@ struct Params {
     int attractor;         // 0 Maxwellian, 1 factorized
     int reduced;           // reduced compressibility (u = j / rho0)
     int has_field;         // per-cell force field present
-    int pair;              // step with two cells of a row per thread (packed FP32, periodic x)
+    int pair;              // step with two cells of a row per thread (packed FP32): 1 = whole warps per row
+                           // (periodic x, nx a multiple of 64), 2 = any row length, x walls included
     int big;               // Q * S >= 2^32: kernels with 64-bit element offsets
     int z0, nzc;           // planes z0 .. z0 + nzc - 1 of a step launch (nzc = 0: all planes)
     long long N;           // cells updated (nx ny nz)
@@ -65,6 +66,9 @@ template <class R> struct PR {
     int bc[3];
     int les, vd, attractor, reduced, has_field;
     int z0;                // first plane of a step launch (blockIdx.z counts from it)
+    // flat launches (flat_len != 0): blockIdx.x counts over the work items of a whole plane, rows
+    // of flat_len items one after another (plane_xy)
+    unsigned flat_len, flat_mul;
     unsigned N;            // cells (also the stride of force and moment fields)
     unsigned S;            // direction-plane stride of a state buffer
     unsigned long long N64, S64;   // the same as 64-bit values (kernels with 64-bit offsets)
@@ -82,6 +86,7 @@ template <class R> inline PR<R> typed(const Params& p) {
     for (int a = 0; a < 3; ++a) q.bc[a] = p.bc[a];
     q.les = p.les; q.vd = p.vd; q.attractor = p.attractor; q.reduced = p.reduced; q.has_field = p.has_field;
     q.z0 = p.z0;
+    q.flat_len = q.flat_mul = 0;
     q.N = (unsigned)p.N;
     q.S = (unsigned)p.S;
     q.N64 = (unsigned long long)p.N;
@@ -99,6 +104,31 @@ template <class R> inline PR<R> typed(const Params& p) {
     q.cs = (R)p.cs; q.vd_aplus = (R)p.vd_aplus; q.vd_utau_nu = (R)p.vd_utau_nu; q.rho0 = (R)p.rho0;
     q.omega_nu = (R)(1.0 / p.tau0);
     return q;
+}
+
+// Flat launches. With a block row per grid row, a row of len items keeps ceil(len / 32) warps
+// busy, the last of them partly: 65 items (nx = 130, two cells per thread) leave a third of three
+// warps idle, and a block that spans several rows idles on all of them. Counting over the plane
+// instead leaves only the plane's last block partly idle. The thread finds its row by a division
+// by the row length, which is one multiplication by flat_mul = ceil(2^32 / len): for n < 2^32 the
+// estimate is the quotient or one more.
+template <class P> inline void set_flat(P& q, int len) {
+    q.flat_len = (unsigned)len;
+    q.flat_mul = (unsigned)(((1ULL << 32) + (unsigned)len - 1) / (unsigned)len);      // len >= 2
+}
+// The item (x, y) of this thread in its plane; false for threads past the end (len items a row)
+template <class P> __device__ __forceinline__ bool plane_xy(const P& p, int len, int& x, int& y) {
+    x = blockIdx.x * blockDim.x + threadIdx.x;
+    y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (p.flat_len != 0) {
+        const unsigned n = (unsigned)x;
+        unsigned r = __umulhi(n, p.flat_mul);
+        if (r * p.flat_len > n) --r;
+        y = (int)r;
+        x = (int)(n - r * p.flat_len);
+        return y < p.ny;
+    }
+    return x < len && y < p.ny;
 }
 
 // Element offsets into state buffers ([Q][S]) and [3][N] fields: 32-bit unsigned while Q * S and

@@ -87,6 +87,19 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S>()) k_step(const S* 
 // inst_pair_*.cu (so that the kernel variants compile in parallel) ----------------------------
 template <class S, class FT>
 void launch_pair(const void* src, void* dst, const void* Ff, const Params& p, cudaStream_t st);
+// the same on rows of any length and with x walls (inst_ragged_*.cu): variants with WALLS only
+template <class S, class FT>
+void launch_pair_ragged(const void* src, void* dst, const void* Ff, const Params& p, cudaStream_t st);
+template <class S, class FT>
+void launch_pair_any(const void* src, void* dst, const void* Ff, const Params& p, cudaStream_t st) {
+    if constexpr (FT::WALLS) {
+        if (p.pair == 2) {
+            launch_pair_ragged<S, FT>(src, dst, Ff, p, st);
+            return;
+        }
+    }
+    launch_pair<S, FT>(src, dst, Ff, p, st);
+}
 
 // ---- density and velocity of the pulled field ----------------------------------------------
 template <int D, class S, bool WALLS, bool BIG = false>
@@ -211,11 +224,11 @@ void launch_step_ft(const void* src, void* dst, const void* Ff, const Params& p,
     using R = typename Codec<S>::R;
     if constexpr (FT::UNIT && D == 3) {     // the D3Q27 UNIT variants are pair-kernel variants
         static_assert(sizeof(R) == 4, "D3Q27 UNIT variants are pair-kernel variants");
-        launch_pair<S, FT>(src, dst, Ff, p, st);
+        launch_pair_any<S, FT>(src, dst, Ff, p, st);
         return;
     } else if constexpr (D == 3 && sizeof(R) == 4) {
         if (p.pair) {
-            launch_pair<S, FT>(src, dst, Ff, p, st);
+            launch_pair_any<S, FT>(src, dst, Ff, p, st);
             return;
         }
     }
@@ -241,9 +254,9 @@ void launch_step_g(const void* src, void* dst, const void* Ff, const Params& p, 
                     // compile time
                     if (simple_collision(p) && (p.attractor != 0) != (p.reduced != 0)) {
                         if (p.attractor != 0)
-                            launch_pair<S, Feat<W, L, false, false, true, false, false, false, true, false>>(src, dst, Ff, p, st);
+                            launch_pair_any<S, Feat<W, L, false, false, true, false, false, false, true, false>>(src, dst, Ff, p, st);
                         else
-                            launch_pair<S, Feat<W, L, false, false, true, false, false, false, false, true>>(src, dst, Ff, p, st);
+                            launch_pair_any<S, Feat<W, L, false, false, true, false, false, false, false, true>>(src, dst, Ff, p, st);
                         return;
                     }
                 }
@@ -359,7 +372,8 @@ cudaError_t launch_step(const void* src, void* dst, const void* Ff, const Params
             return cudaGetLastError();
         }
     }
-    if (has_walls(p)) launch_step_l<D, S, true>(src, dst, Ff, p, st);
+    // the ragged rows have variants with run-time wall tests only
+    if (has_walls(p) || p.pair == 2) launch_step_l<D, S, true>(src, dst, Ff, p, st);
     else launch_step_l<D, S, false>(src, dst, Ff, p, st);
     return cudaGetLastError();
 }

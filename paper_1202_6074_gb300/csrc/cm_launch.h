@@ -38,6 +38,13 @@ constexpr int kReduceMaxBlocks = 1216;
 inline bool pair_eligible(const Params& p, int D, bool fp32_arith) {
     return D == 3 && fp32_arith && p.bc[0] == 0 && p.nx % 64 == 0;
 }
+// The same kernel on any row length, and with x walls: what the automatic choice takes for the
+// other D3Q27 grids with FP32 arithmetic. The line is drawn on the plane (a slab of a grid takes
+// the same kernel as the whole grid, so that their results stay equal bit for bit).
+constexpr int kRaggedPairPlane = 2048;
+inline bool ragged_pair_eligible(const Params& p, int D, bool fp32_arith) {
+    return D == 3 && fp32_arith && !p.big && p.nx >= 8 && (long long)p.nx * p.ny >= kRaggedPairPlane;
+}
 
 // Two steps per pass for FP32 storage (launch_pair_two_steps, inst_pair_tb_f32.cu): planes in
 // groups of kTwoStepGroup, the intermediate state in a ring of kTwoStepRing + 2 planes.

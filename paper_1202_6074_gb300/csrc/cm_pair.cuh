@@ -7,8 +7,10 @@ namespace cm {
 
 // Two cells of a row, (x, y, z) and (x + nx/2, y, z) or the adjacent (x0, y, z) and
 // (x0 + 1, y, z), are updated together with the packed FP32 instructions (R = F2). They share y
-// and z, hence the y/z wall flags, the row offsets, and the van Driest constant; x must be
-// periodic. Each lane is rounded as the scalar FP32 arithmetic rounds it.
+// and z, hence the y/z wall flags, the row offsets, and the van Driest constant. Each lane is
+// rounded as the scalar FP32 arithmetic rounds it. Rows of nx % 64 == 0 cells fill whole warps;
+// other rows are laid end to end over a plane (plane_xy), and an odd row pairs (x, x + (nx+1)/2),
+// its last thread without a second cell of its own.
 #ifndef CM_PAIR_MIN_BLOCKS
 #define CM_PAIR_MIN_BLOCKS 4
 #endif
@@ -83,21 +85,38 @@ struct Ring {
     }
 };
 
+// Half-way bounce-back from a moving wall: d += 6 (e . u_w) for each of the two cells' links of
+// direction i, averaged over the walls a link crosses (see gather_impl)
+template <int i>
+__device__ __forceinline__ void add_wall_motion(const PR<float>& p, bool by, bool bz, bool bA, bool bB, float& da, float& db) {
+    constexpr int a = Lat<3>::ex(i), b = Lat<3>::ey(i), c = Lat<3>::ez(i);
+    float eu = 0.f;
+    if constexpr (b != 0) eu = by ? eu + e_dot<3, i>(p.uw[1][b > 0 ? 0 : 1]) : eu;
+    if constexpr (c != 0) eu = bz ? eu + e_dot<3, i>(p.uw[2][c > 0 ? 0 : 1]) : eu;
+    float eA = eu, eB = eu;
+    if constexpr (a > 0) eA = bA ? eu + e_dot<3, i>(p.uw[0][0]) : eu;      // only the first cell crosses x = -1/2
+    if constexpr (a < 0) eB = bB ? eu + e_dot<3, i>(p.uw[0][1]) : eu;      // only the last one crosses the far wall
+    const int cnt = (int)by + (int)bz;
+    da = fmaf(wall_factor<float>(cnt + (int)bA), eA, da);
+    db = fmaf(wall_factor<float>(cnt + (int)bB), eB, db);
+}
+
 // The pair gathers return the stored deviations d (moving-wall term included), not h = w d:
 // the collision takes them as they are (see collide).
 // RS / RD: the source / destination state is the ring (else a full buffer with stride p.S)
-template <class S, bool WALLS, bool RS = false, bool BIG = false>
-__device__ __forceinline__ void gather_pair(const S* __restrict__ src, int x, int y, int z, const PR<float>& p, F2 (&h)[27],
-                                            const Ring& ring = Ring{}) {
+// WALLS: y or z links may cross a wall; XW: x links may (only the row's first and last cell's)
+template <class S, bool WALLS, bool RS = false, bool BIG = false, bool XW = false>
+__device__ __forceinline__ void gather_pair(const S* __restrict__ src, int x, int xB, int y, int z, const PR<float>& p,
+                                            F2 (&h)[27], const Ring& ring = Ring{}) {
     static_assert(!(RS && BIG), "the plane ring is only used on grids with 32-bit offsets");
     using IX = Ix<BIG>;
     const IX PS = RS ? (IX)ring.stride : plane_stride<BIG>(p);
-    const int half = p.nx >> 1;
+    const bool xoA = XW && p.bc[0] == 1 && x == 0, xoB = XW && p.bc[0] == 1 && xB == p.nx - 1;
     int xa[3], xb[3], ys[3], zs[3];
     bool yo[3] = {false, false, false}, zo[3] = {false, false, false};
 #pragma unroll
     for (int k = 0; k < 3; ++k) {          // slot k <-> e = k - 1, source coordinate = x - e
-        int sa = x + 1 - k, sb = x + half + 1 - k;     // sa in [-1, half], sb in [half - 1, nx]
+        int sa = x + 1 - k, sb = xB + 1 - k;     // sa in [-1, nx - 1], sb in [0, nx]
         if (sa < 0) sa += p.nx;
         if (sb >= p.nx) sb -= p.nx;
         xa[k] = sa;
@@ -131,26 +150,18 @@ __device__ __forceinline__ void gather_pair(const S* __restrict__ src, int x, in
 #pragma unroll
             for (int b = 0; b < 3; ++b) row[c][b] = (unsigned)((zs[c] * p.ny + ys[b]) * p.nx);
     }
-    cellB = cellA + (unsigned)half;
+    cellB = cellA + (unsigned)(xB - x);
     sfor<27>([&](auto I) {
         constexpr int i = decltype(I)::value;
         constexpr int a = Lat<3>::ex(i) + 1, b = Lat<3>::ey(i) + 1, c = Lat<3>::ez(i) + 1;
         const IX base = IX(i) * PS + row[c][b];
-        if constexpr (WALLS) {
-            const bool by = yo[b], bz = zo[c];
-            const bool bounced = by || bz;
+        if constexpr ((WALLS && (b != 1 || c != 1)) || (XW && a != 1)) {
+            const bool by = WALLS && yo[b], bz = WALLS && zo[c];
+            const bool bA = a == 2 && xoA, bB = a == 0 && xoB;      // the links across the x walls
             const IX own = IX(Lat<3>::opp(i)) * PS;
-            float da = Codec<S>::ld(src + (bounced ? own + cellA : base + (unsigned)xa[a]));
-            float db = Codec<S>::ld(src + (bounced ? own + cellB : base + (unsigned)xb[a]));
-            if (p.moving) {       // half-way bounce-back from a moving wall (see gather_impl)
-                constexpr int sy = (b == 2) ? 0 : 1, sz = (c == 2) ? 0 : 1;
-                float eu = 0.f;
-                if constexpr (b != 1) eu = by ? eu + e_dot<3, i>(p.uw[1][sy]) : eu;
-                if constexpr (c != 1) eu = bz ? eu + e_dot<3, i>(p.uw[2][sz]) : eu;
-                const float k = wall_factor<float>((int)by + (int)bz);
-                da = fmaf(k, eu, da);
-                db = fmaf(k, eu, db);
-            }
+            float da = Codec<S>::ld(src + (by || bz || bA ? own + cellA : base + (unsigned)xa[a]));
+            float db = Codec<S>::ld(src + (by || bz || bB ? own + cellB : base + (unsigned)xb[a]));
+            if (p.moving) add_wall_motion<i>(p, by, bz, bA, bB, da, db);
             h[slot<3>(i)] = F2(da, db);
         } else {
             if constexpr (sizeof(S) == 2)   // 64-bit row pointers (measured faster at 16-bit storage)
@@ -165,11 +176,12 @@ __device__ __forceinline__ void gather_pair(const S* __restrict__ src, int x, in
 // buffer. Slot k <-> e_x = k - 1 reads columns x - e_x: c0[k] for the first cell, c1[k] for the
 // second; the e_x = 0 pair (x0, x0 + 1) is one aligned two-entry read (direction-plane
 // strides, row offsets and x0 are even).
-template <class S, bool WALLS, bool BIG = false>
+template <class S, bool WALLS, bool BIG = false, bool XW = false>
 __device__ __forceinline__ void gather_adj(const S* __restrict__ src, int x0, int y, int z, const PR<float>& p,
                                            F2 (&h)[27]) {
     using IX = Ix<BIG>;
     const IX PS = plane_stride<BIG>(p);
+    const bool xoA = XW && p.bc[0] == 1 && x0 == 0, xoB = XW && p.bc[0] == 1 && x0 + 2 == p.nx;
     const int c0[3] = {x0 + 1, x0, x0 == 0 ? p.nx - 1 : x0 - 1};
     const int c1[3] = {x0 + 2 == p.nx ? 0 : x0 + 2, x0 + 1, x0};
     int ys[3], zs[3];
@@ -198,26 +210,18 @@ __device__ __forceinline__ void gather_adj(const S* __restrict__ src, int x0, in
         constexpr int i = decltype(I)::value;
         constexpr int a = Lat<3>::ex(i) + 1, b = Lat<3>::ey(i) + 1, c = Lat<3>::ez(i) + 1;
         const IX base = IX(i) * PS + row[c][b];
-        if constexpr (WALLS) {
-            const bool by = yo[b], bz = zo[c];
-            const bool bounced = by || bz;
+        if constexpr ((WALLS && (b != 1 || c != 1)) || (XW && a != 1)) {
+            const bool by = WALLS && yo[b], bz = WALLS && zo[c];
+            const bool bA = a == 2 && xoA, bB = a == 0 && xoB;      // the links across the x walls
             const IX back = IX(Lat<3>::opp(i)) * PS + own;       // the cells' own reflected entries
             float2 d;
             if constexpr (a == 1) {
-                d = Codec<S>::ld2(src + (bounced ? back : base + (unsigned)x0));
+                d = Codec<S>::ld2(src + (by || bz ? back : base + (unsigned)x0));
             } else {
-                d.x = Codec<S>::ld(src + (bounced ? back : base + (unsigned)c0[a]));
-                d.y = Codec<S>::ld(src + (bounced ? back + 1u : base + (unsigned)c1[a]));
+                d.x = Codec<S>::ld(src + (by || bz || bA ? back : base + (unsigned)c0[a]));
+                d.y = Codec<S>::ld(src + (by || bz || bB ? back + 1u : base + (unsigned)c1[a]));
             }
-            if (p.moving) {       // half-way bounce-back from a moving wall (see gather_impl)
-                constexpr int sy = (b == 2) ? 0 : 1, sz = (c == 2) ? 0 : 1;
-                float eu = 0.f;
-                if constexpr (b != 1) eu = by ? eu + e_dot<3, i>(p.uw[1][sy]) : eu;
-                if constexpr (c != 1) eu = bz ? eu + e_dot<3, i>(p.uw[2][sz]) : eu;
-                const float k = wall_factor<float>((int)by + (int)bz);
-                d.x = fmaf(k, eu, d.x);
-                d.y = fmaf(k, eu, d.y);
-            }
+            if (p.moving) add_wall_motion<i>(p, by, bz, bA, bB, d.x, d.y);
             h[slot<3>(i)] = F2(d.x, d.y);
         } else if constexpr (a == 1) {
             const float2 d = Codec<S>::ld2(src + x0 + base);
@@ -264,48 +268,74 @@ __device__ __forceinline__ void gather_adj_inner(const S* __restrict__ src, int 
     });
 }
 
-template <class S, class FT, bool RS = false, bool RD = false, bool ADJ = false>
+// RAG: rows of any length (laid end to end over the blocks, plane_xy) and walls across x. A
+// variant of its own: the few instructions more cost the 16-bit steps of whole-warp rows 2.5 %.
+// Against the one-cell kernel, which these grids ran before (per step of a 50-step run): a cavity
+// 130 x 111 x 90 FP32 79.6 -> 56.7 us, the factorized attractor 150 x 97 x 75 FP16 47.3 -> 35.1 us.
+template <class S, class FT, bool RS = false, bool RD = false, bool ADJ = false, bool RAG = false>
 __global__ void __launch_bounds__(kBlock, pair_min_blocks<S, FT>()) k_step_pair(const S* __restrict__ src, S* __restrict__ dst,
                                                                           const float* __restrict__ Ff, PR<float> p,
                                                                           Ring ring) {
-    const int half = p.nx >> 1;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const int half = RAG ? (p.nx + 1) >> 1 : p.nx >> 1;            // pairs per row
+    int x, y;
     const int z = (int)blockIdx.z + ring.z0;     // the ring's group, or the launch's first plane
-    if (x >= half || y >= p.ny) return;
+    // the warp pulls across no x edge: it holds no row's first or last pair (ADJ)
+    bool inner = false;
+    if constexpr (RAG) {
+        const bool valid = plane_xy(p, half, x, y);
+        if constexpr (ADJ && FT::FX) inner = __all_sync(0xffffffffu, x > 0 && 2 * x + 2 < p.nx);
+        if (!valid) return;
+    } else {
+        x = blockIdx.x * blockDim.x + threadIdx.x;
+        y = blockIdx.y * blockDim.y + threadIdx.y;
+        if (x >= half || y >= p.ny) return;
+        // warps are 32 consecutive threads of one row (blockDim.x is a multiple of 32): the warp
+        // covers columns 2 x_w .. 2 x_w + 63 (the test is warp-uniform)
+        const int xw = x - (int)(threadIdx.x & 31u);
+        inner = ADJ && FT::FX && xw > 0 && 2 * (xw + 31) + 2 < p.nx;
+    }
+    static_assert(!RAG || (!RS && !RD && !FT::BIG), "ragged rows only between full state buffers, 32-bit offsets");
     static_assert(!ADJ || (!RS && !RD), "adjacent cells only between full state buffers");
-    // global cells (force field) and the destination cells
+    // global cells (force field) and the destination cells; the last thread of an odd row has no
+    // second cell: it updates the row's last cell once more, without storing it
     const int xa = ADJ ? 2 * x : x;
-    const unsigned cellA = (unsigned)((z * p.ny + y) * p.nx + xa), cellB = cellA + (ADJ ? 1u : (unsigned)half);
-    const unsigned dA = RD ? ring.plane(z) + (unsigned)(y * p.nx + x) : cellA, dB = dA + (unsigned)half;
+    const bool second = !RAG || ADJ || x + half < p.nx;
+    const int xb = ADJ ? xa + 1 : second ? x + half : p.nx - 1;
+    const unsigned cellA = (unsigned)((z * p.ny + y) * p.nx + xa), cellB = cellA + (unsigned)(xb - xa);
+    const unsigned dA = RD ? ring.plane(z) + (unsigned)(y * p.nx + x) : cellA, dB = dA + (unsigned)(xb - xa);
     static_assert(!FT::BIG || (!RS && !RD), "the plane ring is only used on grids with 32-bit offsets");
     using IX = Ix<FT::BIG>;
     const IX PS = RD ? (IX)ring.stride : plane_stride<FT::BIG>(p);
     F2 h[27];
+    // walls across y or z: the cells next to one (uniform over most warps) take the wall-aware pull.
+    // Walls across x: on a row of 130 cells every warp holds a row's first or last cell, so all
+    // cells pull through the form that selects between the neighbour and the reflected entry for
+    // the two lanes concerned (18 selects) instead of diverging.
+    bool near = false;
+    if constexpr (FT::WALLS)
+        near = (p.bc[1] == 1 && (y == 0 || y == p.ny - 1)) || (p.bc[2] == 1 && (z == 0 || z == p.nz - 1));
+    constexpr bool XW = FT::WALLS && RAG;      // the other variants have periodic x
     if constexpr (ADJ) {
-        // warps are 32 consecutive threads of one row (blockDim.x is a multiple of 32): the warp
-        // covers columns 2 x_w .. 2 x_w + 63, and pulls across the periodic x edge only if it holds
-        // the row's first or last pair (the test is warp-uniform). The immediate-offset gather of
-        // such interior warps measured +1.5 % for the FX channel variant, but -7 % for the 512^3
-        // force-field LES and -2.3 % for the unforced Taylor-Green step, which keep gather_adj.
-        const int xw = x - (int)(threadIdx.x & 31u);
-        const bool inner = FT::FX && xw > 0 && 2 * (xw + 31) + 2 < p.nx;
-        bool near = false;
-        if constexpr (FT::WALLS)
-            near = (p.bc[1] == 1 && (y == 0 || y == p.ny - 1)) || (p.bc[2] == 1 && (z == 0 || z == p.nz - 1));
+        // The immediate-offset gather of interior warps measured +1.5 % for the FX channel variant,
+        // but -7 % for the 512^3 force-field LES and -2.3 % for the unforced Taylor-Green step,
+        // which keep gather_adj.
         if (near) {
-            if constexpr (FT::WALLS) gather_adj<S, true, FT::BIG>(src, xa, y, z, p, h);
+            if constexpr (FT::WALLS) gather_adj<S, true, FT::BIG, XW>(src, xa, y, z, p, h);
         } else if (inner) {
             if constexpr (FT::FX) gather_adj_inner<S, FT::BIG>(src, xa, y, z, p, h);
+        } else if (XW && p.bc[0] == 1) {
+            if constexpr (XW) gather_adj<S, false, FT::BIG, true>(src, xa, y, z, p, h);
         } else {
             gather_adj<S, false, FT::BIG>(src, xa, y, z, p, h);
         }
-    } else if constexpr (FT::WALLS) {
-        const bool near = (p.bc[1] == 1 && (y == 0 || y == p.ny - 1)) || (p.bc[2] == 1 && (z == 0 || z == p.nz - 1));
-        if (near) gather_pair<S, true, RS, FT::BIG>(src, x, y, z, p, h, ring);
-        else gather_pair<S, false, RS, FT::BIG>(src, x, y, z, p, h, ring);
     } else {
-        gather_pair<S, false, RS, FT::BIG>(src, x, y, z, p, h, ring);
+        if (near) {
+            if constexpr (FT::WALLS) gather_pair<S, true, RS, FT::BIG, XW>(src, x, xb, y, z, p, h, ring);
+        } else if (XW && p.bc[0] == 1) {
+            if constexpr (XW) gather_pair<S, false, RS, FT::BIG, true>(src, x, xb, y, z, p, h, ring);
+        } else {
+            gather_pair<S, false, RS, FT::BIG>(src, x, xb, y, z, p, h, ring);
+        }
     }
     F2 F[3];
     if (FT::FIELD && p.has_field) {
@@ -333,10 +363,10 @@ __global__ void __launch_bounds__(kBlock, pair_min_blocks<S, FT>()) k_step_pair(
             Codec<S>::st2(dst + dA + (size_t)PS * i, v.v.x, v.v.y);
         } else if constexpr (sizeof(S) == 2) {
             Codec<S>::st(dst + dA + (size_t)PS * i, v.v.x);
-            Codec<S>::st(dst + dB + (size_t)PS * i, v.v.y);
+            if (second) Codec<S>::st(dst + dB + (size_t)PS * i, v.v.y);
         } else {
             Codec<S>::st(dst + (IX(i) * PS + dA), v.v.x);
-            Codec<S>::st(dst + (IX(i) * PS + dB), v.v.y);
+            if (second) Codec<S>::st(dst + (IX(i) * PS + dB), v.v.y);
         }
     });
 }
@@ -359,6 +389,26 @@ void launch_pair(const void* src, void* dst, const void* Ff, const Params& p, cu
         }
     }
     k_step_pair<S, FT><<<g, b, 0, st>>>((const S*)src, (S*)dst, (const float*)Ff, typed<float>(p), planes);
+}
+
+// The same on rows of any length (Params::pair == 2). Adjacent cells also need even rows.
+template <class S, class FT>
+void launch_pair_ragged(const void* src, void* dst, const void* Ff, const Params& p, cudaStream_t st) {
+    const int half = (p.nx + 1) / 2;
+    PR<float> q = typed<float>(p);
+    set_flat(q, half);
+    const dim3 g((unsigned)(((long long)half * p.ny + kBlock - 1) / kBlock), 1, step_planes(p));
+    Ring planes{};
+    planes.z0 = p.z0;
+    if constexpr (pair_adjacent<S, FT>()) {
+        const uintptr_t two = 2 * sizeof(S);
+        if (p.nx % 2 == 0 && (uintptr_t)src % two == 0 && (uintptr_t)dst % two == 0) {
+            k_step_pair<S, FT, false, false, true, true><<<g, kBlock, 0, st>>>((const S*)src, (S*)dst, (const float*)Ff, q,
+                                                                               planes);
+            return;
+        }
+    }
+    k_step_pair<S, FT, false, false, false, true><<<g, kBlock, 0, st>>>((const S*)src, (S*)dst, (const float*)Ff, q, planes);
 }
 
 // Two steps per pass (temporal blocking through the L2 cache). Steps t -> t+1 -> t+2 from the
@@ -402,6 +452,28 @@ int launch_pair_two_steps(const void* A, void* C, void* ring, int P, int slots, 
     }
     return launches;
 }
+
+// every feature combination of the ragged rows (one per eddy viscosity and force field; the wall
+// tests stay at run time, so that the library builds half as many variants)
+#define CM_RAGGED(S, ...) \
+    template void launch_pair_ragged<S, Feat<true, __VA_ARGS__>>(const void*, void*, const void*, const Params&, cudaStream_t);
+#define CM_RAGGED_INSTANTIATE(S)                                                                             \
+    CM_RAGGED(S, false, false, false) CM_RAGGED(S, false, true, false)                                       \
+    CM_RAGGED(S, true, false, false) CM_RAGGED(S, true, true, false)                                         \
+    CM_RAGGED(S, false, false, false, true) CM_RAGGED(S, true, false, false, true)                           \
+    CM_RAGGED(S, false, false, false, true, false, false, false, true, false)                                \
+    CM_RAGGED(S, true, false, false, true, false, false, false, true, false)                                 \
+    CM_RAGGED(S, false, false, false, true, false, false, false, false, true)                                \
+    CM_RAGGED(S, true, false, false, true, false, false, false, false, true)
+#define CM_RAGGED_INSTANTIATE_UNIT(S)                                                                        \
+    CM_RAGGED(S, false, false, false, false, true) CM_RAGGED(S, false, true, false, false, true)             \
+    CM_RAGGED(S, true, false, false, false, true) CM_RAGGED(S, true, true, false, false, true)               \
+    CM_RAGGED(S, false, false, false, false, true, false, true) CM_RAGGED(S, true, false, false, false, true, false, true)
+#define CM_RAGGED_INSTANTIATE_GEN(S)                                                                         \
+    CM_RAGGED(S, false, false, true) CM_RAGGED(S, false, true, true)                                         \
+    CM_RAGGED(S, true, false, true) CM_RAGGED(S, true, true, true)                                           \
+    CM_RAGGED(S, false, false, true, false, true) CM_RAGGED(S, false, true, true, false, true)               \
+    CM_RAGGED(S, true, false, true, false, true) CM_RAGGED(S, true, true, true, false, true)
 
 // every feature combination the dispatcher in cm_kernels.cuh can pass
 #define CM_PAIR_INSTANTIATE(S)                                                                              \

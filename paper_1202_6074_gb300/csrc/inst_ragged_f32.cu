@@ -1,0 +1,6 @@
+// Two-cells-per-thread step kernels on rows of any length, float storage: the standard collision and the unforced forms.
+#include "cm_pair.cuh"
+
+namespace cm {
+CM_RAGGED_INSTANTIATE(float)
+}  // namespace cm

@@ -1,0 +1,6 @@
+// Two-cells-per-thread step kernels on rows of any length, __half storage: the general forms.
+#include "cm_pair.cuh"
+
+namespace cm {
+CM_RAGGED_INSTANTIATE_GEN(__half)
+}  // namespace cm

@@ -1,0 +1,6 @@
+// Two-cells-per-thread step kernels on rows of any length, float storage: the forced collision with unit higher-order rates.
+#include "cm_pair.cuh"
+
+namespace cm {
+CM_RAGGED_INSTANTIATE_UNIT(float)
+}  // namespace cm
