@@ -46,6 +46,7 @@ struct Params {
     int pair;              // step with two cells of a row per thread (packed FP32): 1 = whole warps per row
                            // (periodic x, nx a multiple of 64), 2 = any row length, x walls included
     int big;               // Q * S >= 2^32: kernels with 64-bit element offsets
+    int chain;             // launch as a dependent of the kernel before it (chain_wait)
     int z0, nzc;           // planes z0 .. z0 + nzc - 1 of a step launch (nzc = 0: all planes)
     long long N;           // cells updated (nx ny nz)
     long long S;           // elements between direction planes of a state buffer (N, or nx ny (nz + 2) on a slab)
@@ -105,6 +106,14 @@ template <class R> inline PR<R> typed(const Params& p) {
     q.omega_nu = (R)(1.0 / p.tau0);
     return q;
 }
+
+// Chained launches: the steps captured into one graph follow each other as programmatic
+// dependents. A step's blocks are dispatched as soon as all blocks of the step before have
+// started and slots come free, work out their coordinates, and wait here until that step has
+// completed and its stores are visible; no global memory is read or written before the wait. A
+// kernel launched any other way passes both at once.
+__device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Flat launches. With a block row per grid row, a row of len items keeps ceil(len / 32) warps
 // busy, the last of them partly: 65 items (nx = 130, two cells per thread) leave a third of three

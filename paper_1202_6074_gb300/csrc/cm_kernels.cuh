@@ -33,6 +33,21 @@ inline dim3 cell_grid(const Params& p, dim3 b) {
     return dim3((p.nx + b.x - 1) / b.x, (p.ny + b.y - 1) / b.y, step_planes(p));
 }
 
+// launch of a step kernel: with p.chain as a programmatic dependent of the kernel before it
+template <class... P, class... A>
+inline void launch_chained(const Params& p, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = p.chain ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 template <class R, bool FIELD = true, bool BIG = false>
 __device__ __forceinline__ void load_force(const R* __restrict__ Ff, const PR<R>& p, unsigned cell, R F[3]) {
     if (FIELD && p.has_field) {
@@ -67,7 +82,9 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S>()) k_step(const S* 
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = (int)blockIdx.z + p.z0;
+    chain_begin();
     if (x >= p.nx || y >= p.ny) return;
+    chain_wait();
     using IX = Ix<FT::BIG>;
     const unsigned cell = (unsigned)((z * p.ny + y) * p.nx + x);
     const IX PS = plane_stride<FT::BIG>(p);
@@ -235,7 +252,7 @@ void launch_step_ft(const void* src, void* dst, const void* Ff, const Params& p,
     // small grids: one warp per block so that the few blocks spread over as many SMs as possible
     // (the step is latency bound there; 128-thread blocks would leave most SMs idle)
     const dim3 b = p.N <= kSmallGrid ? dim3(CM_SMALL_BLOCK, 1, 1) : cell_block(p.nx), g = cell_grid(p, b);
-    k_step<D, S, FT><<<g, b, 0, st>>>((const S*)src, (S*)dst, (const R*)Ff, typed<R>(p));
+    launch_chained(p, k_step<D, S, FT>, g, b, st, (const S*)src, (S*)dst, (const R*)Ff, typed<R>(p));
 }
 
 // no force anywhere and unit rates above second order (the SIMPLE variant applies)
@@ -320,8 +337,8 @@ void launch_step_big_g(const void* src, void* dst, const void* Ff, const Params&
         launch_pair<S, Feat<W, L, F, true, false, false, true>>(src, dst, Ff, p, st);
     } else {
         const dim3 b = cell_block(p.nx), g = cell_grid(p, b);
-        k_step<3, S, Feat<W, L, F, true, false, false, true>><<<g, b, 0, st>>>((const S*)src, (S*)dst, (const R*)Ff,
-                                                                            typed<R>(p));
+        launch_chained(p, k_step<3, S, Feat<W, L, F, true, false, false, true>>, g, b, st, (const S*)src, (S*)dst,
+                       (const R*)Ff, typed<R>(p));
     }
 }
 template <class S>

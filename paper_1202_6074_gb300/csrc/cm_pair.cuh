@@ -276,6 +276,7 @@ template <class S, class FT, bool RS = false, bool RD = false, bool ADJ = false,
 __global__ void __launch_bounds__(kBlock, pair_min_blocks<S, FT>()) k_step_pair(const S* __restrict__ src, S* __restrict__ dst,
                                                                           const float* __restrict__ Ff, PR<float> p,
                                                                           Ring ring) {
+    chain_begin();
     const int half = RAG ? (p.nx + 1) >> 1 : p.nx >> 1;            // pairs per row
     int x, y;
     const int z = (int)blockIdx.z + ring.z0;     // the ring's group, or the launch's first plane
@@ -306,6 +307,7 @@ __global__ void __launch_bounds__(kBlock, pair_min_blocks<S, FT>()) k_step_pair(
     static_assert(!FT::BIG || (!RS && !RD), "the plane ring is only used on grids with 32-bit offsets");
     using IX = Ix<FT::BIG>;
     const IX PS = RD ? (IX)ring.stride : plane_stride<FT::BIG>(p);
+    chain_wait();
     F2 h[27];
     // walls across y or z: the cells next to one (uniform over most warps) take the wall-aware pull.
     // Walls across x: on a row of 130 cells every warp holds a row's first or last cell, so all
@@ -383,12 +385,12 @@ void launch_pair(const void* src, void* dst, const void* Ff, const Params& p, cu
     if constexpr (pair_adjacent<S, FT>()) {
         const uintptr_t two = 2 * sizeof(S);
         if ((uintptr_t)src % two == 0 && (uintptr_t)dst % two == 0) {
-            k_step_pair<S, FT, false, false, true><<<g, b, 0, st>>>((const S*)src, (S*)dst, (const float*)Ff,
-                                                                     typed<float>(p), planes);
+            launch_chained(p, k_step_pair<S, FT, false, false, true>, g, b, st, (const S*)src, (S*)dst, (const float*)Ff,
+                           typed<float>(p), planes);
             return;
         }
     }
-    k_step_pair<S, FT><<<g, b, 0, st>>>((const S*)src, (S*)dst, (const float*)Ff, typed<float>(p), planes);
+    launch_chained(p, k_step_pair<S, FT>, g, b, st, (const S*)src, (S*)dst, (const float*)Ff, typed<float>(p), planes);
 }
 
 // The same on rows of any length (Params::pair == 2). Adjacent cells also need even rows.
@@ -403,12 +405,13 @@ void launch_pair_ragged(const void* src, void* dst, const void* Ff, const Params
     if constexpr (pair_adjacent<S, FT>()) {
         const uintptr_t two = 2 * sizeof(S);
         if (p.nx % 2 == 0 && (uintptr_t)src % two == 0 && (uintptr_t)dst % two == 0) {
-            k_step_pair<S, FT, false, false, true, true><<<g, kBlock, 0, st>>>((const S*)src, (S*)dst, (const float*)Ff, q,
-                                                                               planes);
+            launch_chained(p, k_step_pair<S, FT, false, false, true, true>, g, kBlock, st, (const S*)src, (S*)dst,
+                           (const float*)Ff, q, planes);
             return;
         }
     }
-    k_step_pair<S, FT, false, false, false, true><<<g, kBlock, 0, st>>>((const S*)src, (S*)dst, (const float*)Ff, q, planes);
+    launch_chained(p, k_step_pair<S, FT, false, false, false, true>, g, kBlock, st, (const S*)src, (S*)dst,
+                   (const float*)Ff, q, planes);
 }
 
 // Two steps per pass (temporal blocking through the L2 cache). Steps t -> t+1 -> t+2 from the
