@@ -775,6 +775,158 @@ template <class R, int a, int b, int c> __device__ __forceinline__ R weight_cm(c
     return k;
 }
 
+// omega_nu: 1 / tau0, or the effective rate of the Smagorinsky model from the non-equilibrium
+// stress P = {xx, yy, zz, xy, xz, yz}
+template <class R, class FT>
+__device__ __forceinline__ R shear_rate(const R (&P)[6], R irho, const PR<scalar_t<R>>& p, scalar_t<R> cs_eff) {
+    using T = scalar_t<R>;
+    if constexpr (FT::LES) {
+        R tau = R(p.tau0);
+        if (cs_eff > T(0)) {
+            R Q2 = P[0] * P[0];
+            Q2 = fma(P[1], P[1], Q2);
+            Q2 = fma(P[2], P[2], Q2);
+            R O2 = P[3] * P[3];
+            O2 = fma(P[4], P[4], O2);
+            O2 = fma(P[5], P[5], O2);
+            const R Qn = les_sqrt(fma(R(2), O2, Q2));
+            // tau_eff = (tau + sqrt(tau^2 + 18 sqrt(2) C^2 |Pi| / rho)) / 2
+            const R k = R(T(25.455844122715710878) * cs_eff * cs_eff);
+            tau = R(0.5) * (tau + les_sqrt(fma(tau, tau, k * Qn * irho)));
+        }
+        return les_rcp(tau);
+    } else if constexpr (std::is_same_v<R, double>) {
+        // the same value as the reciprocal below (both IEEE-rounded), without an FP64 division
+        // per cell on GB300's narrow FP64 pipe; the FP32 forms keep the per-thread reciprocal,
+        // which measured faster there (register allocation of the 16-bit steps)
+        return R(p.omega_nu);
+    } else {
+        return rcp(R(p.tau0));
+    }
+}
+
+// ------------------------------------------------------------------------------------------
+// The unforced collision with omega_3 = omega_4 = 1 (SIMPLE) in the Maxwellian's product form.
+//
+// With no source and unit rates above second order the post-collision state is the Maxwellian plus
+// the relaxed non-equilibrium stress T, so neither the full forward transform nor the inverse
+// transform of 27 moments is needed:
+//   in:  rho, j and the raw second-order moments are sums of the x-line moments, and
+//        P_ab = R_ab - c_s^2 drho delta_ab - u_a j_b  (j = rho u: no force)
+//   out: f / w = rho phi(u_x) phi(u_y) phi(u_z) + sum of the six T_ab times products of the 1D
+//        populations g_k of a unit k-th central moment (divided by the 1D weight):
+//        phi = 1 + eta;  eta: e = 0: -3/2 u^2,  e = +-1: 3 u^2 +- 3 u
+//        g_0: e = 0: 3/2 + eta, +-1: eta;  g_1: e = 0: -3 u, +-1: 6 u +- 3;  g_2: -3/2, 3
+//        evaluated line by line along x: with E = rho phi_y phi_z - 1, E' = E + its T part of x order
+//        0, M = 3 x that of order 1, S = E + 3 x that of order 2 and V = 1 + E':
+//        t1 = 3 u V + M,  t2 = 3 u^2 V + 2 u M + S,  d_+- = t2 +- t1,  d_0 = 3/2 E' - t2 / 2
+// Everything stays a deviation from the rest state. About 310 operations a cell instead of the 416
+// of the two transforms (packed, D3Q27), which the 16-bit steps are bound by: Taylor-Green 256^3
+// BF16 SIMPLETIME us a step. The FP32 steps stay bound by HBM.
+// Out: the post-collision deviations d = h / w (slot order).
+// ------------------------------------------------------------------------------------------
+template <int D, class R, class FT>
+__device__ __forceinline__ void collide_simple(R (&m)[Lat<D>::Q], const PR<scalar_t<R>>& p, scalar_t<R> cs_eff) {
+    using T = scalar_t<R>;
+    static_assert(FT::SIMPLE && !FT::FACT && !FT::RED, "the product form is the unforced Maxwellian one");
+    constexpr int NZ = Lat<D>::NZ;
+    const R C = R((T)moment_scale<D>());
+    const R third = R(T(1) / 3);
+    raw_x<D, R>(m);
+    // sums over the lines of one e_z with the weights (1, 4, 1) of e_y: raw moments of order
+    // (x, y) = 00 (A), 01 (Y), 02 (Q), 10 (B), 11 (W), 20 (X)
+    R A[NZ], Y[NZ], Q[NZ], B[NZ], W[NZ], X[NZ];
+#pragma unroll
+    for (int c = 0; c < NZ; ++c) {
+        const int l0 = 9 * c, l1 = l0 + 3, l2 = l0 + 6;      // e_y = -1, 0, +1
+        Q[c] = m[l0] + m[l2];
+        A[c] = fma(R(4), m[l1], Q[c]);
+        Y[c] = m[l2] - m[l0];
+        B[c] = fma(R(4), m[l1 + 1], m[l0 + 1] + m[l2 + 1]);
+        W[c] = m[l2 + 1] - m[l0 + 1];
+        X[c] = fma(R(4), m[l1 + 2], m[l0 + 2] + m[l2 + 2]);
+    }
+    auto over_z = [&](const R (&v)[NZ]) -> R {
+        if constexpr (D == 3) return fma(R(4), v[1], v[0] + v[2]);
+        else return v[0];
+    };
+    const R drho = over_z(A) * C, jx = over_z(B) * C, jy = over_z(Y) * C;
+    const R rho = R(1) + drho, irho = rcp(rho);
+    const R cd = drho * R(T(-1) / 3);
+    const R ux = jx * irho, uy = jy * irho;
+    R P[6];
+    P[0] = fma(-ux, jx, fma(over_z(X), C, cd));
+    P[1] = fma(-uy, jy, fma(over_z(Q), C, cd));
+    P[2] = R(0);
+    P[3] = fma(-ux, jy, over_z(W) * C);
+    P[4] = P[5] = R(0);
+    R uz = R(0);
+    if constexpr (D == 3) {
+        const R jz = (A[2] - A[0]) * C;
+        uz = jz * irho;
+        P[2] = fma(-uz, jz, fma(A[0] + A[2], C, cd));
+        P[4] = fma(-ux, jz, (B[2] - B[0]) * C);
+        P[5] = fma(-uy, jz, (Y[2] - Y[0]) * C);
+    }
+    const R wnu = shear_rate<R, FT>(P, irho, p, cs_eff);
+    const R wb = (p.omega_bulk > T(0)) ? R(p.omega_bulk) : wnu;
+    const R omn = R(1) - wnu;
+    const R corr = (wnu - wb) * (P[0] + P[1] + P[2]) * R(T(1) / D);
+    const R Txx = fma(omn, P[0], corr), Tyy = fma(omn, P[1], corr), Tzz = fma(omn, P[2], corr);
+    const R Txy = omn * P[3], Txz = omn * P[4], Tyz = omn * P[5];
+
+    // 1D populations over the 1D weights, index e + 1
+    auto tables = [&](R u, R (&eta)[3], R (&g0)[3], R (&g1)[3]) {
+        const R q = u * u, u3 = u * R(3), q3 = q * R(3);
+        eta[1] = q * R(-1.5);
+        eta[0] = q3 - u3;
+        eta[2] = q3 + u3;
+        g0[0] = eta[0];
+        g0[1] = eta[1] + R(1.5);
+        g0[2] = eta[2];
+        const R u6 = u3 + u3;
+        g1[0] = u6 - R(3);
+        g1[1] = -u3;
+        g1[2] = u6 + R(3);
+    };
+    R ey[3], y0[3], y1[3];
+    tables(uy, ey, y0, y1);
+    const R tx = ux + ux, x3 = ux * R(3), qx3 = ux * x3;
+    auto x_line = [&](int l, R E, R Ep, R M, R S) {
+        const R V = Ep + R(1);
+        const R t1 = fma(x3, V, M);
+        const R t2 = fma(qx3, V, fma(tx, M, S));
+        m[3 * l] = t2 - t1;
+        m[3 * l + 1] = fma(R(-0.5), t2, Ep * R(1.5));
+        m[3 * l + 2] = t2 + t1;
+    };
+    const R Txx3 = Txx * R(3), Txy3 = Txy * R(3);
+    const R yy[3] = {Tyy * R(3), Tyy * R(-1.5), Tyy * R(3)};       // T_yy g_2(y)
+    if constexpr (D == 3) {
+        R ez[3], z0[3], z1[3];
+        tables(uz, ez, z0, z1);
+        const R Txz3 = Txz * R(3);
+        const R zz[3] = {Tzz * R(3), Tzz * R(-1.5), Tzz * R(3)};   // T_zz g_2(z)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const R phi = R(1) + ey[b], yz1 = Tyz * y1[b], xy1 = Txy3 * y1[b], xx0 = Txx3 * y0[b], xz0 = Txz3 * y0[b];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const R E = fma(rho, fma(phi, ez[c], ey[b]), drho);
+                const R Ep = fma(yy[b], z0[c], fma(y0[b], zz[c], fma(yz1, z1[c], E)));
+                const R M = fma(xy1, z0[c], xz0 * z1[c]);
+                x_line(3 * c + b, E, Ep, M, fma(xx0, z0[c], E));
+            }
+        }
+    } else {
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const R E = fma(rho, ey[b], drho);
+            x_line(b, E, E + yy[b], Txy3 * y1[b], fma(Txx3, y0[b], E));
+        }
+    }
+}
+
 // ------------------------------------------------------------------------------------------
 // The collision in central-moment space (generic form; see the file header and cmlbm.h).
 // In: the stored deviations d = h / w (slot order; h = fbar - w), force F, the eddy-viscosity
@@ -789,6 +941,11 @@ template <int D, class R, class FT, bool DEV = false>
 __device__ __forceinline__ void collide(R (&m)[Lat<D>::Q], const R F[3], const PR<scalar_t<R>>& p, scalar_t<R> cs_eff) {
     using T = scalar_t<R>;
     constexpr int Q = Lat<D>::Q;
+    if constexpr (FT::SIMPLE && !FT::FACT && !FT::RED) {
+        static_assert(DEV, "the product form returns the deviations");
+        collide_simple<D, R, FT>(m, p, cs_eff);
+        return;
+    }
     raw_x<D, R>(m);
     const Hydro<D, R> hy = hydro_x<D, R, FT::GEN, !FT::SIMPLE, !FT::FX, FT::RED>(m, F, p);
     const R drho = hy.drho, rho = R(1) + hy.drho, ndrho = -hy.drho;
@@ -829,30 +986,7 @@ __device__ __forceinline__ void collide(R (&m)[Lat<D>::Q], const R F[3], const P
         Pyz = fma(m[midx(0, 1, 1)], C, u[1] * u[2]);
     }
 
-    R wnu;
-    if constexpr (FT::LES) {
-        R tau = R(p.tau0);
-        if (cs_eff > T(0)) {
-            R Q2 = Pxx * Pxx;
-            Q2 = fma(Pyy, Pyy, Q2);
-            Q2 = fma(Pzz, Pzz, Q2);
-            R O2 = Pxy * Pxy;
-            O2 = fma(Pxz, Pxz, O2);
-            O2 = fma(Pyz, Pyz, O2);
-            const R Qn = les_sqrt(fma(R(2), O2, Q2));
-            // tau_eff = (tau + sqrt(tau^2 + 18 sqrt(2) C^2 |Pi| / rho)) / 2
-            const R k = R(T(25.455844122715710878) * cs_eff * cs_eff);
-            tau = R(0.5) * (tau + les_sqrt(fma(tau, tau, k * Qn * irho)));
-        }
-        wnu = les_rcp(tau);
-    } else if constexpr (std::is_same_v<R, double>) {
-        // the same value as the reciprocal below (both IEEE-rounded), without an FP64 division
-        // per cell on GB300's narrow FP64 pipe; the FP32 forms keep the per-thread reciprocal,
-        // which measured faster there (register allocation of the 16-bit steps)
-        wnu = R(p.omega_nu);
-    } else {
-        wnu = rcp(R(p.tau0));
-    }
+    const R wnu = shear_rate<R, FT>({Pxx, Pyy, Pzz, Pxy, Pxz, Pyz}, irho, p, cs_eff);
     const R wb = (p.omega_bulk > T(0)) ? R(p.omega_bulk) : wnu;
 
     // kappa of f at second order, used by the source recursion (sigma = 0 at second order)

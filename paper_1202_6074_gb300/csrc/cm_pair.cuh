@@ -59,7 +59,9 @@ template <class S, class FT> constexpr bool pair_adjacent() { return sizeof(S) =
 // collision takes the stored deviations either way). The 16-bit steps, which are bound by
 // their FP32 arithmetic, fold (the force-field LES BF16 step: +2.2 % at 512^3); the FP32 steps,
 // bound by HBM, keep the product at the store.
-template <class S, class FT> __host__ __device__ constexpr bool pair_dev() { return sizeof(S) == 2; }
+template <class S, class FT> __host__ __device__ constexpr bool pair_dev() {
+    return sizeof(S) == 2 || (FT::SIMPLE && !FT::FACT && !FT::RED);      // the product form has no other output
+}
 
 // Blocks of kBlock threads whose x extent divides the pair threads of a row (a multiple of 32:
 // nx is a multiple of 64 on this kernel), so that no block is left partly idle at the end of a
