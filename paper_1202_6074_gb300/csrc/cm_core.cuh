@@ -223,8 +223,8 @@ template <class R> using scalar_t = typename Scalar<R>::T;
 // gives at unit rates, with its multiplications by 1 - omega and omega left out); with GEN the
 // attractor is the factorized one where the parameters select it.
 // FX: a UNIT collision whose force is uniform with F_y = F_z = 0 (a flow driven along x, as in
-// a channel): the source recursion keeps only its x terms, and the moments without an x
-// exponent get no source. The same values as UNIT (the terms left out are products with zero).
+// a channel): the source recursion acts along x only, and the collision is evaluated in product form
+// (collide_product).
 // BIG: 64-bit element offsets (grids with Q * S >= 2^32).
 // FACT / RED: the factorized attractor (Sec. 13) / reduced compressibility (Sec. 12) fixed at
 // compile time instead of read from the parameters as GEN does (for SIMPLE collisions, the
@@ -239,6 +239,11 @@ struct Feat {
     static_assert(!FX_ || (UNIT_ && !FIELD_ && !GEN_), "FX is a UNIT collision with a uniform force along x");
     static_assert(!(FACT_ || RED_) || (SIMPLE_ && !GEN_), "FACT / RED are SIMPLE collisions of one form");
 };
+
+// the variants whose collision is evaluated in product form (collide_product)
+template <class FT> __host__ __device__ constexpr bool product_form() {
+    return (FT::SIMPLE && !FT::FACT && !FT::RED) || FT::FX;
+}
 
 // ------------------------------------------------------------------------------------------
 // Lattices
@@ -606,7 +611,7 @@ template <int D, class R> __device__ __forceinline__ void raw_x(R (&m)[Lat<D>::Q
 // rho - 1 and the momentum (Eqs. densitycalculation, velocitycalculation) from the x-line
 // moments of raw_x(): line l = (e_y + 1) + 3 (e_z + 1) carries the weight r1(e_y) r1(e_z), so
 // the sums over e_y (per e_z) and then over e_z are again multiply-adds by 4
-template <int D, class R, bool GEN = true, bool FORCED = true, bool FYZ = true, bool RED = false>
+template <int D, class R, bool GEN = true, bool FORCED = true, bool RED = false>
 __device__ __forceinline__ Hydro<D, R> hydro_x(const R (&m)[Lat<D>::Q], const R F[3], const PR<scalar_t<R>>& p) {
     using T = scalar_t<R>;
     constexpr int NZ = Lat<D>::NZ;
@@ -637,8 +642,8 @@ __device__ __forceinline__ Hydro<D, R> hydro_x(const R (&m)[Lat<D>::Q], const R 
     o.drho = drho;
     if constexpr (FORCED) {
         o.jx = fma(R(0.5), F[0], jx);
-        o.jy = FYZ ? fma(R(0.5), F[1], jy) : jy;
-        o.jz = FYZ ? fma(R(0.5), F[2], jz) : jz;
+        o.jy = fma(R(0.5), F[1], jy);
+        o.jz = fma(R(0.5), F[2], jz);
     } else {
         o.jx = jx;
         o.jy = jy;
@@ -806,29 +811,43 @@ __device__ __forceinline__ R shear_rate(const R (&P)[6], R irho, const PR<scalar
 }
 
 // ------------------------------------------------------------------------------------------
-// The unforced collision with omega_3 = omega_4 = 1 (SIMPLE) in the Maxwellian's product form.
+// The collision with omega_3 = omega_4 = 1 and no force (SIMPLE) or a uniform force along x (FX), in
+// the Maxwellian's product form.
 //
-// With no source and unit rates above second order the post-collision state is the Maxwellian plus
-// the relaxed non-equilibrium stress T, so neither the full forward transform nor the inverse
-// transform of 27 moments is needed:
-//   in:  rho, j and the raw second-order moments are sums of the x-line moments, and
-//        P_ab = R_ab - c_s^2 drho delta_ab - u_a j_b  (j = rho u: no force)
+// At unit rates above second order the post-collision state is the Maxwellian, plus the relaxed
+// non-equilibrium stress T, plus half the source sigma; neither the full forward transform nor the
+// inverse transform of 27 moments is needed:
+//   in:  rho, R = sum f e and the raw second-order moments are sums of the x-line moments; with
+//        rho u = R + F / 2,  P_xx = R_xx - c_s^2 drho - u_x (R_x - F/2),  P_xa = R_xa - u_a R_x,
+//        P_ab = R_ab - c_s^2 drho delta_ab - u_a R_b for a, b = y, z
 //   out: f / w = rho phi(u_x) phi(u_y) phi(u_z) + sum of the six T_ab times products of the 1D
 //        populations g_k of a unit k-th central moment (divided by the 1D weight):
 //        phi = 1 + eta;  eta: e = 0: -3/2 u^2,  e = +-1: 3 u^2 +- 3 u
 //        g_0: e = 0: 3/2 + eta, +-1: eta;  g_1: e = 0: -3 u, +-1: 6 u +- 3;  g_2: -3/2, 3
-//        evaluated line by line along x: with E = rho phi_y phi_z - 1, E' = E + its T part of x order
-//        0, M = 3 x that of order 1, S = E + 3 x that of order 2 and V = 1 + E':
-//        t1 = 3 u V + M,  t2 = 3 u^2 V + 2 u M + S,  d_+- = t2 +- t1,  d_0 = 3/2 E' - t2 / 2
-// Everything stays a deviation from the rest state. About 310 operations a cell instead of the 416
-// of the two transforms (packed, D3Q27), which the 16-bit steps are bound by: Taylor-Green 256^3
-// BF16 SIMPLETIME us a step. The FP32 steps stay bound by HBM.
+//   source: with F along x the recursion sigma_abc = a (F/rho) kappa_(a-1)bc, kappa = kappabar + sigma/2
+//        acts on the x exponent alone (and gives the conserved moments their values: kappa_x = 0,
+//        sigma_x = F, no second order), so it needs no y or z transform: per x-line, with the line's
+//        moments N_0 = sum f, N_1 = sum f (e_x - u_x) before the collision (over the line's weight),
+//        half the source is (F/2rho) N_0 at x order 1 and (F/rho) (N_1 + (F/2rho) N_0) at order 2.
+// Evaluated line by line along x: with E = rho phi_y phi_z - 1, E' = E + its T part of x order 0,
+// M = the T part and source of order 1, S = E + 3 x those of order 2 and V = 1 + E':
+//   r1 = u V + M,  t2 = 3 u^2 V + 6 u M + S,  d_+- = t2 +- 3 r1,  d_0 = 3/2 E' - t2 / 2
+// COMP (FP32 storage): u = j / rho is rounded, and rho u then misses the momentum by the same
+// relative error in every direction at once. The residual K = j - rho u (exact, one fma) goes in as
+// the first-order central moment it is: M += K_x, and 3 K / rho beside 3 u in eta of y and z before
+// their one rounding. Without it the error of an FP32 run against 64 bits grew by a third
+// (Couette 1500 x 701, 100 steps); 16-bit storage rounds a thousand times coarser.
+// Everything stays a deviation from the rest state. About 310 operations a cell (350 with the force)
+// instead of the 416 (540) of the two transforms (D3Q27), which the 16-bit steps and FP64 are bound
+// by. Measured, against the transforms, per step: Taylor-Green 256^3 BF16 316 -> 304 us, D2Q9 1500 x
+// 701 FP32 10.9 -> 10.2 us; with a force along x, D3Q27 128^3 FP64 2.4 -> 1.4 ms, D2Q9 64 x 32 FP64
+// 6.6 -> 5.6 us. The FP32 D3Q27 steps stay bound by HBM.
 // Out: the post-collision deviations d = h / w (slot order).
 // ------------------------------------------------------------------------------------------
-template <int D, class R, class FT>
-__device__ __forceinline__ void collide_simple(R (&m)[Lat<D>::Q], const PR<scalar_t<R>>& p, scalar_t<R> cs_eff) {
+template <int D, class R, class FT, bool COMP>
+__device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const PR<scalar_t<R>>& p, scalar_t<R> cs_eff) {
     using T = scalar_t<R>;
-    static_assert(FT::SIMPLE && !FT::FACT && !FT::RED, "the product form is the unforced Maxwellian one");
+    static_assert(product_form<FT>(), "the product form is the Maxwellian one at unit rates");
     constexpr int NZ = Lat<D>::NZ;
     const R C = R((T)moment_scale<D>());
     const R third = R(T(1) / 3);
@@ -850,22 +869,27 @@ __device__ __forceinline__ void collide_simple(R (&m)[Lat<D>::Q], const PR<scala
         if constexpr (D == 3) return fma(R(4), v[1], v[0] + v[2]);
         else return v[0];
     };
-    const R drho = over_z(A) * C, jx = over_z(B) * C, jy = over_z(Y) * C;
+    const R drho = over_z(A) * C, Rx = over_z(B) * C, jy = over_z(Y) * C;
     const R rho = R(1) + drho, irho = rcp(rho);
     const R cd = drho * R(T(-1) / 3);
+    R jx = Rx, Rm = Rx;                  // j_x = R_x + F / 2, R_x - F / 2
+    if constexpr (FT::FX) {
+        jx = fma(R(0.5), Fx, Rx);
+        Rm = fma(R(-0.5), Fx, Rx);
+    }
     const R ux = jx * irho, uy = jy * irho;
     R P[6];
-    P[0] = fma(-ux, jx, fma(over_z(X), C, cd));
+    P[0] = fma(-ux, Rm, fma(over_z(X), C, cd));
     P[1] = fma(-uy, jy, fma(over_z(Q), C, cd));
     P[2] = R(0);
-    P[3] = fma(-ux, jy, over_z(W) * C);
+    P[3] = fma(-uy, Rx, over_z(W) * C);
     P[4] = P[5] = R(0);
-    R uz = R(0);
+    R uz = R(0), jz = R(0);
     if constexpr (D == 3) {
-        const R jz = (A[2] - A[0]) * C;
+        jz = (A[2] - A[0]) * C;
         uz = jz * irho;
         P[2] = fma(-uz, jz, fma(A[0] + A[2], C, cd));
-        P[4] = fma(-ux, jz, (B[2] - B[0]) * C);
+        P[4] = fma(-uz, Rx, (B[2] - B[0]) * C);
         P[5] = fma(-uy, jz, (Y[2] - Y[0]) * C);
     }
     const R wnu = shear_rate<R, FT>(P, irho, p, cs_eff);
@@ -876,45 +900,70 @@ __device__ __forceinline__ void collide_simple(R (&m)[Lat<D>::Q], const PR<scala
     const R Txy = omn * P[3], Txz = omn * P[4], Tyz = omn * P[5];
 
     // 1D populations over the 1D weights, index e + 1
-    auto tables = [&](R u, R (&eta)[3], R (&g0)[3], R (&g1)[3]) {
-        const R q = u * u, u3 = u * R(3), q3 = q * R(3);
+    auto tables = [&](R u, R j, R (&eta)[3], R (&g0)[3], R (&g1)[3]) {
+        const R q = u * u, q3 = q * R(3);
+        R lo = q3, hi = q3;
+        if constexpr (COMP) {
+            const R k = fma(-rho, u, j) * (irho * R(3));
+            lo = q3 - k;
+            hi = q3 + k;
+        }
         eta[1] = q * R(-1.5);
-        eta[0] = q3 - u3;
-        eta[2] = q3 + u3;
+        eta[0] = fma(R(-3), u, lo);
+        eta[2] = fma(R(3), u, hi);
         g0[0] = eta[0];
         g0[1] = eta[1] + R(1.5);
         g0[2] = eta[2];
-        const R u6 = u3 + u3;
-        g1[0] = u6 - R(3);
-        g1[1] = -u3;
-        g1[2] = u6 + R(3);
+        g1[0] = fma(R(6), u, R(-3));
+        g1[1] = u * R(-3);
+        g1[2] = fma(R(6), u, R(3));
     };
     R ey[3], y0[3], y1[3];
-    tables(uy, ey, y0, y1);
-    const R tx = ux + ux, x3 = ux * R(3), qx3 = ux * x3;
+    tables(uy, jy, ey, y0, y1);
+    const R x6 = ux * R(6), qx3 = ux * ux * R(3);
+    R Kx = R(0);
+    if constexpr (COMP) Kx = fma(-rho, ux, jx);
+    // the source: M += s10 + s11 m_0, S += s20 + s21 m_0 + s22 m_1 with the weighted line moments
+    // m_0, m_1 of raw_x() (N_0 = 1 + m_0 / 6, N_1 = m_1 / 6 - u_x N_0)
+    R s10, s11, s20, s21, s22;
+    if constexpr (FT::FX) {
+        const R Fr = Fx * irho, Fh = Fr * R(0.5);
+        s10 = COMP ? Fh + Kx : Fh;
+        s11 = Fh * R(T(1) / 6);
+        const R f = Fr * (Fh - ux);
+        s20 = f * R(3);
+        s21 = f * R(0.5);
+        s22 = Fh;
+    }
     auto x_line = [&](int l, R E, R Ep, R M, R S) {
+        if constexpr (FT::FX) {
+            M = fma(s11, m[3 * l], M);
+            S = fma(s22, m[3 * l + 1], fma(s21, m[3 * l], S + s20));
+        }
         const R V = Ep + R(1);
-        const R t1 = fma(x3, V, M);
-        const R t2 = fma(qx3, V, fma(tx, M, S));
-        m[3 * l] = t2 - t1;
+        const R r1 = fma(ux, V, M);
+        const R t2 = fma(qx3, V, fma(x6, M, S));
+        m[3 * l] = fma(R(-3), r1, t2);
         m[3 * l + 1] = fma(R(-0.5), t2, Ep * R(1.5));
-        m[3 * l + 2] = t2 + t1;
+        m[3 * l + 2] = fma(R(3), r1, t2);
     };
-    const R Txx3 = Txx * R(3), Txy3 = Txy * R(3);
+    constexpr bool M0 = FT::FX || COMP;          // a part of M common to all lines
+    R m0 = Kx;
+    if constexpr (FT::FX) m0 = s10;
+    const R Txx3 = Txx * R(3);
     const R yy[3] = {Tyy * R(3), Tyy * R(-1.5), Tyy * R(3)};       // T_yy g_2(y)
     if constexpr (D == 3) {
         R ez[3], z0[3], z1[3];
-        tables(uz, ez, z0, z1);
-        const R Txz3 = Txz * R(3);
+        tables(uz, jz, ez, z0, z1);
         const R zz[3] = {Tzz * R(3), Tzz * R(-1.5), Tzz * R(3)};   // T_zz g_2(z)
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const R phi = R(1) + ey[b], yz1 = Tyz * y1[b], xy1 = Txy3 * y1[b], xx0 = Txx3 * y0[b], xz0 = Txz3 * y0[b];
+            const R phi = R(1) + ey[b], yz1 = Tyz * y1[b], xy1 = Txy * y1[b], xx0 = Txx3 * y0[b], xz0 = Txz * y0[b];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 const R E = fma(rho, fma(phi, ez[c], ey[b]), drho);
                 const R Ep = fma(yy[b], z0[c], fma(y0[b], zz[c], fma(yz1, z1[c], E)));
-                const R M = fma(xy1, z0[c], xz0 * z1[c]);
+                const R M = fma(xy1, z0[c], M0 ? fma(xz0, z1[c], m0) : xz0 * z1[c]);
                 x_line(3 * c + b, E, Ep, M, fma(xx0, z0[c], E));
             }
         }
@@ -922,7 +971,7 @@ __device__ __forceinline__ void collide_simple(R (&m)[Lat<D>::Q], const PR<scala
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
             const R E = fma(rho, ey[b], drho);
-            x_line(b, E, E + yy[b], Txy3 * y1[b], fma(Txx3, y0[b], E));
+            x_line(b, E, E + yy[b], M0 ? fma(Txy, y1[b], m0) : Txy * y1[b], fma(Txx3, y0[b], E));
         }
     }
 }
@@ -937,17 +986,17 @@ __device__ __forceinline__ void collide_simple(R (&m)[Lat<D>::Q], const PR<scala
 // R is the arithmetic type (double, float, or F2 for two cells of one row; cs_eff and the
 // parameters are then scalars shared by both cells).
 // ------------------------------------------------------------------------------------------
-template <int D, class R, class FT, bool DEV = false>
+template <int D, class R, class FT, bool DEV = false, bool COMP = false>
 __device__ __forceinline__ void collide(R (&m)[Lat<D>::Q], const R F[3], const PR<scalar_t<R>>& p, scalar_t<R> cs_eff) {
     using T = scalar_t<R>;
     constexpr int Q = Lat<D>::Q;
-    if constexpr (FT::SIMPLE && !FT::FACT && !FT::RED) {
+    if constexpr (product_form<FT>()) {
         static_assert(DEV, "the product form returns the deviations");
-        collide_simple<D, R, FT>(m, p, cs_eff);
+        collide_product<D, R, FT, COMP>(m, F[0], p, cs_eff);
         return;
     }
     raw_x<D, R>(m);
-    const Hydro<D, R> hy = hydro_x<D, R, FT::GEN, !FT::SIMPLE, !FT::FX, FT::RED>(m, F, p);
+    const Hydro<D, R> hy = hydro_x<D, R, FT::GEN, !FT::SIMPLE, FT::RED>(m, F, p);
     const R drho = hy.drho, rho = R(1) + hy.drho, ndrho = -hy.drho;
     const R u[3] = {hy.ux, hy.uy, hy.uz};
     central_forward_from_x<D, R>(m, u[0], u[1], u[2]);
@@ -962,8 +1011,8 @@ __device__ __forceinline__ void collide(R (&m)[Lat<D>::Q], const R F[3], const P
         if constexpr (D == 3) m[midx(0, 0, 1)] = fma(ndrho, u[2], hy.jz);
     } else {
         m[midx(1, 0, 0)] = fma(ndrho, u[0], fma(R(0.5), F[0], hy.jx));
-        m[midx(0, 1, 0)] = fma(ndrho, u[1], FT::FX ? hy.jy : fma(R(0.5), F[1], hy.jy));
-        if constexpr (D == 3) m[midx(0, 0, 1)] = fma(ndrho, u[2], FT::FX ? hy.jz : fma(R(0.5), F[2], hy.jz));
+        m[midx(0, 1, 0)] = fma(ndrho, u[1], fma(R(0.5), F[1], hy.jy));
+        if constexpr (D == 3) m[midx(0, 0, 1)] = fma(ndrho, u[2], fma(R(0.5), F[2], hy.jz));
     }
 
     const R third = R(T(1) / 3);
@@ -1069,14 +1118,12 @@ __device__ __forceinline__ void collide(R (&m)[Lat<D>::Q], const R F[3], const P
                     constexpr int a = ex_a(t), b = ex_b(t), c = ex_c(t);
                     R s = R(0);
                     if constexpr (a > 0) s = fma(a == 2 ? Fr2[0] : Fr[0], kap[t - 1], s);
-                    if constexpr (b > 0 && !FT::FX) s = fma(b == 2 ? Fr2[1] : Fr[1], kap[t - 3], s);
-                    if constexpr (c > 0 && !FT::FX) s = fma(c == 2 ? Fr2[2] : Fr[2], kap[t - 9], s);
-                    constexpr bool sourced = a > 0 || (!FT::FX && (b > 0 || c > 0));
+                    if constexpr (b > 0) s = fma(b == 2 ? Fr2[1] : Fr[1], kap[t - 3], s);
+                    if constexpr (c > 0) s = fma(c == 2 ? Fr2[2] : Fr[2], kap[t - 9], s);
                     const R hs = R(0.5) * s;
                     const R kw = weight_cm<R, a, b, c>(cw);
                     if constexpr (ord(t) < 2 * D) {
-                        if constexpr (sourced) kap[t] = fma(R(0.5), s, fma(m[t], C, kw));
-                        else kap[t] = fma(m[t], C, kw);
+                        kap[t] = fma(R(0.5), s, fma(m[t], C, kw));
                     }
                     constexpr bool even = (a % 2 == 0) && (b % 2 == 0) && (c % 2 == 0);
                     constexpr int twos = (a == 2) + (b == 2) + (c == 2);
@@ -1092,8 +1139,7 @@ __device__ __forceinline__ void collide(R (&m)[Lat<D>::Q], const R F[3], const P
                         // halving is exact). The standard collision writes it as one packed fma; the
                         // general forms keep the product and the sum, which measured fewer spills
                         // there (0-24 B against 16-44 B at 128 registers, FP32)
-                        if constexpr (!sourced) m[t] = DM;
-                        else if constexpr (FT::GEN) m[t] = DM + hs;
+                        if constexpr (FT::GEN) m[t] = DM + hs;
                         else m[t] = fma(R(0.5), s, DM);
                     } else {
                         const R w = (ord(t) == 3) ? w3 : w4;

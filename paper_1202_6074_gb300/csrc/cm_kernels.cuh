@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S>()) k_step(const S* 
     R F[3];
     load_force<R, FT::FIELD, FT::BIG>(Ff, p, cell, F);
     // the collision returns the stored deviations (inverse weights folded into its last sweep)
-    collide<D, R, FT, true>(h, F, p, smagorinsky_constant<R, FT::LES>(p, y));
+    collide<D, R, FT, true, sizeof(S) == 4>(h, F, p, smagorinsky_constant<R, FT::LES>(p, y));
     sfor<Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
         Codec<S>::st(dst + (IX(i) * PS + cell), h[slot<D>(i)]);
@@ -239,7 +239,7 @@ inline bool has_walls(const Params& p) { return p.bc[0] == 1 || p.bc[1] == 1 || 
 template <int D, class S, class FT>
 void launch_step_ft(const void* src, void* dst, const void* Ff, const Params& p, cudaStream_t st) {
     using R = typename Codec<S>::R;
-    if constexpr (FT::UNIT && D == 3) {     // the D3Q27 UNIT variants are pair-kernel variants
+    if constexpr (FT::UNIT && !FT::FX && D == 3) {     // these D3Q27 variants are pair-kernel variants
         static_assert(sizeof(R) == 4, "D3Q27 UNIT variants are pair-kernel variants");
         launch_pair_any<S, FT>(src, dst, Ff, p, st);
         return;
@@ -259,6 +259,12 @@ void launch_step_ft(const void* src, void* dst, const void* Ff, const Params& p,
 inline bool simple_collision(const Params& p) {
     return !p.has_field && p.F[0] == 0.0 && p.F[1] == 0.0 && p.F[2] == 0.0 && p.omega3 == 1.0 && p.omega4 == 1.0;
 }
+
+// The one-cell kernel takes the product form of a uniform force along x on planes of at least
+// this many cells (as the two-cell kernel does on any it runs on). On smaller ones a step is launch and
+// latency; they keep the transforms, with which a force along x and the same force as a field give
+// the same bits.
+constexpr long long kProductPlane = 2048;
 
 template <int D, class S, bool W, bool L, bool F>
 void launch_step_g(const void* src, void* dst, const void* Ff, const Params& p, cudaStream_t st) {
@@ -290,14 +296,16 @@ void launch_step_g(const void* src, void* dst, const void* Ff, const Params& p, 
             return;
         }
     }
+    if constexpr (!F) {
+        // uniform force along x only
+        if (p.F[1] == 0.0 && p.F[2] == 0.0 && p.omega3 == 1.0 && p.omega4 == 1.0 &&
+            (p.pair || (long long)p.nx * p.ny >= kProductPlane)) {
+            launch_step_ft<D, S, Feat<W, L, false, false, false, true, false, true>>(src, dst, Ff, p, st);
+            return;
+        }
+    }
     if constexpr (D == 3 && sizeof(R) == 4) {
         if (p.pair && p.omega3 == 1.0 && p.omega4 == 1.0) {
-            if constexpr (!F) {
-                if (p.F[1] == 0.0 && p.F[2] == 0.0) {      // uniform force along x only
-                    launch_step_ft<D, S, Feat<W, L, false, false, false, true, false, true>>(src, dst, Ff, p, st);
-                    return;
-                }
-            }
             launch_step_ft<D, S, Feat<W, L, F, false, false, true>>(src, dst, Ff, p, st);
             return;
         }

@@ -19,7 +19,7 @@ namespace cm {
 // allow:
 //   6 blocks (at most 80 registers) for the unforced SIMPLE collision: +2 % over 5, while 7
 //     (72 registers, a 76-byte spill) lose 3 %;
-//   6 for the uniform force along x (FX): +1.5 % over 5;
+//   5 (at most 96) for the uniform force along x (FX): +1 % over 4, while 6 spill over 200 bytes;
 //   5 (at most 96) for the other forced steps without a force field (+5 % on the channel) and
 //     for the UNIT collision with a force field (+1.6 % on the isotropic turbulence LES; at 6
 //     it would spill over 200 bytes).
@@ -27,7 +27,7 @@ namespace cm {
 // registers), as do the general forms (they spill twice as much at 5) and all FP32 steps (the
 // forced FP32 LES loses 7 % at 5).
 #ifndef CM_PAIR_FX_BLOCKS
-#define CM_PAIR_FX_BLOCKS (CM_PAIR_MIN_BLOCKS + 2)
+#define CM_PAIR_FX_BLOCKS (CM_PAIR_MIN_BLOCKS + 1)
 #endif
 #ifndef CM_PAIR_SIMPLE_BLOCKS
 #define CM_PAIR_SIMPLE_BLOCKS (CM_PAIR_MIN_BLOCKS + 2)
@@ -60,7 +60,7 @@ template <class S, class FT> constexpr bool pair_adjacent() { return sizeof(S) =
 // their FP32 arithmetic, fold (the force-field LES BF16 step: +2.2 % at 512^3); the FP32 steps,
 // bound by HBM, keep the product at the store.
 template <class S, class FT> __host__ __device__ constexpr bool pair_dev() {
-    return sizeof(S) == 2 || (FT::SIMPLE && !FT::FACT && !FT::RED);      // the product form has no other output
+    return sizeof(S) == 2 || product_form<FT>();      // the product form has no other output
 }
 
 // Blocks of kBlock threads whose x extent divides the pair threads of a row (a multiple of 32:
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kBlock, pair_min_blocks<S, FT>()) k_step_pair(
         for (int d = 0; d < 3; ++d) F[d] = F2(p.F[d]);
     }
     constexpr bool DEV = pair_dev<S, FT>();
-    collide<3, F2, FT, DEV>(h, F, p, smagorinsky_constant<float, FT::LES>(p, y));
+    collide<3, F2, FT, DEV, sizeof(S) == 4>(h, F, p, smagorinsky_constant<float, FT::LES>(p, y));
     sfor<27>([&](auto I) {
         constexpr int i = decltype(I)::value;
         const F2 v = DEV ? h[slot<3>(i)] : h[slot<3>(i)] * F2((float)inv_weight_scaled<3>(i));
