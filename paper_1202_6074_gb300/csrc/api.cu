@@ -426,6 +426,7 @@ int cmlbm_create(const cmlbm_config* cfg, cmlbm_t** out) {
         return fail(nullptr, CMLBM_ERR_NOMEM, "cudaMalloc of the reduction buffers failed");
     }
     if (cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess) h->nsm = 1;
+    p.nsm = h->nsm;
     if ((c.kernel == CMLBM_KERNEL_AUTO || big) && cm::pair_eligible(p, h->D, c.storage != CMLBM_F64)) p.pair = 1;
     else if (c.kernel == CMLBM_KERNEL_AUTO && cm::ragged_pair_eligible(p, h->D, c.storage != CMLBM_F64)) p.pair = 2;
     const bool two_ok = cm::two_steps_eligible(p, h->D, c.storage == CMLBM_F32, slab);

@@ -45,6 +45,7 @@ struct Params {
     int has_field;         // per-cell force field present
     int pair;              // step with two cells of a row per thread (packed FP32): 1 = whole warps per row
                            // (periodic x, nx a multiple of 64), 2 = any row length, x walls included
+    int nsm;               // multiprocessors of the device
     int big;               // Q * S >= 2^32: kernels with 64-bit element offsets
     int chain;             // launch as a dependent of the kernel before it (chain_wait)
     int z0, nzc;           // planes z0 .. z0 + nzc - 1 of a step launch (nzc = 0: all planes)

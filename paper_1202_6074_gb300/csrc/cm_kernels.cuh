@@ -35,10 +35,12 @@ inline dim3 cell_grid(const Params& p, dim3 b) {
 
 // launch of a step kernel: with p.chain as a programmatic dependent of the kernel before it
 template <class... P, class... A>
-inline void launch_chained(const Params& p, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+inline void launch_chained_smem(const Params& p, void (*kernel)(P...), dim3 grid, dim3 block, int smem, cudaStream_t st,
+                                A... args) {
     cudaLaunchConfig_t c = {};
     c.gridDim = grid;
     c.blockDim = block;
+    c.dynamicSmemBytes = smem;
     c.stream = st;
     cudaLaunchAttribute at = {};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -46,6 +48,10 @@ inline void launch_chained(const Params& p, void (*kernel)(P...), dim3 grid, dim
     c.attrs = &at;
     c.numAttrs = p.chain ? 1 : 0;
     cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+template <class... P, class... A>
+inline void launch_chained(const Params& p, void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+    launch_chained_smem(p, kernel, grid, block, 0, st, args...);
 }
 
 template <class R, bool FIELD = true, bool BIG = false>

@@ -375,6 +375,21 @@ __global__ void __launch_bounds__(kBlock, pair_min_blocks<S, FT>()) k_step_pair(
     });
 }
 
+// k_step_async (cm_async.cuh) takes the 16-bit steps in product form and those with a force field on
+// grids that give every resident warp eight tiles of 64 cells or more (sixty with a force field);
+// below that a warp has too few tiles to copy ahead in. Unforced BF16, us a step, k_step_pair
+// against k_step_async: 64^3 5.3 / 6.5, 128 x 96 x 64 13.2 / 16.1, 128 x 128 x 96 30.6 / 30.2, 192^3
+// 132 / 121; a force along x: 128 x 96 x 96 28.0 / 26.8; a force field: 192 x 160 x 128 97.2 / 99.3,
+// 256 x 192 x 192 226.4 / 225.2, 512^3 3180 / 3100. src must be aligned to its 16-byte copies. The lane
+// arithmetic is the same: so are the bits.
+template <class S, class FT> constexpr bool async_variant() {
+    return sizeof(S) == 2 && (product_form<FT>() || (FT::FIELD && FT::UNIT && !FT::GEN));
+}
+template <class FT> __host__ __device__ constexpr int async_blocks();
+template <class FT> inline int async_resident_warps(const Params& p) { return p.nsm * async_blocks<FT>() * (kBlock / 32); }
+template <class S, class FT>
+void launch_async(const void* src, void* dst, const void* Ff, const Params& p, cudaStream_t st);
+
 template <class S, class FT>
 void launch_pair(const void* src, void* dst, const void* Ff, const Params& p, cudaStream_t st) {
     const int half = p.nx / 2;
@@ -382,6 +397,13 @@ void launch_pair(const void* src, void* dst, const void* Ff, const Params& p, cu
     const dim3 g((half + b.x - 1) / b.x, (p.ny + b.y - 1) / b.y, step_planes(p));
     Ring planes{};
     planes.z0 = p.z0;
+    if constexpr (async_variant<S, FT>()) {
+        const long long tiles = (long long)(p.nx / 64) * p.ny * step_planes(p);
+        if (tiles >= (FT::FIELD ? 60 : 8) * async_resident_warps<FT>(p) && (uintptr_t)src % 16 == 0 && (uintptr_t)dst % 4 == 0) {
+            launch_async<S, FT>(src, dst, Ff, p, st);
+            return;
+        }
+    }
     // adjacent cells need both buffers aligned to two entries (buffers passed in by the caller
     // may be offset); the force field is the library's own allocation
     if constexpr (pair_adjacent<S, FT>()) {

@@ -1,5 +1,5 @@
 // Two-cells-per-thread step kernels for __half storage (see cm_pair.cuh).
-#include "cm_pair.cuh"
+#include "cm_async.cuh"
 
 namespace cm {
 CM_PAIR_INSTANTIATE(__half)

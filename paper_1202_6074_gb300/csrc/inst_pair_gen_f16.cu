@@ -1,5 +1,5 @@
 // Two-cells-per-thread step kernels of the general collision forms for __half storage (see cm_pair.cuh).
-#include "cm_pair.cuh"
+#include "cm_async.cuh"
 
 namespace cm {
 CM_PAIR_INSTANTIATE_GEN(__half)

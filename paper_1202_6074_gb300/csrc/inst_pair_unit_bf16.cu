@@ -1,5 +1,5 @@
 // Two-cells-per-thread step kernels of the forced collision with unit higher-order rates for __nv_bfloat16 storage (see cm_pair.cuh).
-#include "cm_pair.cuh"
+#include "cm_async.cuh"
 
 namespace cm {
 CM_PAIR_INSTANTIATE_UNIT(__nv_bfloat16)
