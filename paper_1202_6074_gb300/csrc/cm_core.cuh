@@ -702,12 +702,11 @@ __device__ __forceinline__ void central_forward_from_x(R (&m)[Lat<D>::Q], R ux, 
 // Inverse sweeps: central moments about u -> populations (slot order). Every sweep leaves out
 // the halving of f-+ = (r2 -+ r1) / 2 (inv1x2), so that the x-line l = (e_y + 1) + 3 (e_z + 1)
 // arrives scaled by 2^k, k = |e_y| + |e_z|. What the last (x) sweep returns, by OUT:
-//   kInvPlain:  the populations h (its constants carry 1/2 and 2^-k);
-//   kInvDev:    the deviations d = h / w (the inverse weights folded into those constants);
+//   kInvDev:    the deviations d = h / w (its constants carry 1/2, 2^-k and the inverse weights);
 //   kInvScaled: 2^n h with n = |e_x| + |e_y| + |e_z| (no constants at all), for a caller that
 //               multiplies every population by a constant anyway (inv_weight_scaled below).
 // Each is bitwise the result of halving in every sweep (a power of two commutes with rounding).
-enum { kInvPlain = 0, kInvDev = 1, kInvScaled = 2 };
+enum { kInvDev = 1, kInvScaled = 2 };
 template <int D, class R, int OUT>
 __device__ __forceinline__ void central_inverse_impl(R (&m)[Lat<D>::Q], R ux, R uy, R uz) {
     using T = scalar_t<R>;
@@ -729,9 +728,7 @@ __device__ __forceinline__ void central_inverse_impl(R (&m)[Lat<D>::Q], R ux, R 
             constexpr int l = decltype(LI)::value;
             constexpr int k = (l % 3 != 1) + (l / 3 != 1 && D == 3);
             constexpr double sk = k == 0 ? 1.0 : k == 1 ? 0.5 : 0.25;
-            constexpr bool dev = OUT == kInvDev;
-            constexpr T he = (T)((dev ? 0.5 / weight_slot<D>(3 * l) : 0.5) * sk),
-                        i0 = (T)((dev ? 1.0 / weight_slot<D>(3 * l + 1) : 1.0) * sk);
+            constexpr T he = (T)(0.5 / weight_slot<D>(3 * l) * sk), i0 = (T)(1.0 / weight_slot<D>(3 * l + 1) * sk);
             const R m0 = m[3 * l], m1 = m[3 * l + 1], m2 = m[3 * l + 2];
             const R r1 = fma(ux, m0, m1);
             const R r2 = fma(qx, m0, fma(tx, m1, m2));
@@ -743,11 +740,6 @@ __device__ __forceinline__ void central_inverse_impl(R (&m)[Lat<D>::Q], R ux, R 
         });
     }
 }
-template <int D, class R>
-__device__ __forceinline__ void central_inverse(R (&m)[Lat<D>::Q], R ux, R uy, R uz) {
-    central_inverse_impl<D, R, kInvPlain>(m, ux, uy, uz);
-}
-
 // The constant that turns the collision's output for direction i (2^n h, see collide) into the
 // stored deviation d = h / w: 1 / (2^n w_i), n = |e_x| + |e_y| + |e_z|.
 template <int D> __host__ __device__ constexpr double inv_weight_scaled(int i) {
@@ -1165,35 +1157,56 @@ __device__ __forceinline__ void collide(R (&m)[Lat<D>::Q], const R F[3], const P
     central_inverse_impl<D, R, DEV ? kInvDev : kInvScaled>(m, u[0], u[1], u[2]);
 }
 
-// Equilibrium deviations fbar - w for (rho, u, F): central moments kappa^M - sigma^M / 2 about u
+// The initial deviations d = fbar / w - 1 for (rho, u, F): central moments kappa^M - sigma^M / 2 about
+// u. The Maxwellian is a product of 1D populations phi = 1 + eta, and the only moments of sigma^M, those
+// with one exponent 1 and the others even, are F_x g_1(x) phi_y phi_z and its like (the tables of
+// collide_product): three multiply-adds a population, and three more with a force, instead of 27
+// moments and their inverse transform.
 template <int D, class R>
-__device__ __forceinline__ void equilibrium(R (&m)[Lat<D>::Q], R rho, R ux, R uy, R uz, const R F[3]) {
-    constexpr int Q = Lat<D>::Q;
-    const R u[3] = {ux, uy, uz};
-    const R q[3] = {ux * ux, uy * uy, uz * uz};
-    const R cw[3][3] = {{R(1), -u[0], R(1) / 3 + q[0]},
-                        {R(1), -u[1], R(1) / 3 + q[1]},
-                        {R(1), -u[2], R(1) / 3 + q[2]}};
+__device__ __forceinline__ void equilibrium(R (&d)[Lat<D>::Q], R rho, R ux, R uy, R uz, const R F[3]) {
     const R drho = rho - R(1);
-    sfor<Q>([&](auto TI) {
-        constexpr int t = decltype(TI)::value;
-        constexpr int a = ex_a(t), b = ex_b(t), c = ex_c(t);
-        constexpr bool even = (a % 2 == 0) && (b % 2 == 0) && (c % 2 == 0);
-        constexpr int twos = (a == 2) + (b == 2) + (c == 2);
-        constexpr R tp = (R)third_pow(twos);
-        // sigma^M by the identity on the Maxwellian moments: non-zero only for one odd axis
-        R s = 0;
-        if constexpr (a == 1 && (b % 2 == 0) && (c % 2 == 0)) s += F[0] * tp;
-        if constexpr (b == 1 && (a % 2 == 0) && (c % 2 == 0)) s += F[1] * tp;
-        if constexpr (c == 1 && (a % 2 == 0) && (b % 2 == 0)) s += F[2] * tp;
-        const R kw = cw[0][a] * cw[1][b] * cw[2][c];
-        R DM;
-        if constexpr (ord(t) == 0) DM = drho;
-        else if constexpr (even) DM = drho * tp - excess<R, a == 2, b == 2, c == 2>(q);
-        else DM = -kw;
-        m[t] = DM - R(0.5) * s;
-    });
-    central_inverse<D, R>(m, u[0], u[1], u[2]);
+    const R u[3] = {ux, uy, uz};
+    R eta[3][3];
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        const R q = u[k] * u[k], q3 = q * R(3);
+        eta[k][0] = fma(R(-3), u[k], q3);
+        eta[k][1] = q * R(-1.5);
+        eta[k][2] = fma(R(3), u[k], q3);
+    }
+    const bool forced = F[0] != R(0) || F[1] != R(0) || F[2] != R(0);
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const R A = fma(R(1) + eta[0][a], eta[1][b], eta[0][a]);      // phi_x phi_y - 1
+#pragma unroll
+            for (int c = 0; c < Lat<D>::NZ; ++c) {
+                if constexpr (D == 3) d[a + 3 * b + 9 * c] = fma(rho, fma(R(1) + A, eta[2][c], A), drho);
+                else d[a + 3 * b] = fma(rho, A, drho);
+            }
+        }
+    if (!forced) return;
+    R g[3][3];                      // -F_k / 2 times g_1 of axis k
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        const R h = F[k] * R(-0.5);
+        g[k][0] = h * fma(R(6), u[k], R(-3));
+        g[k][1] = h * (u[k] * R(-3));
+        g[k][2] = h * fma(R(6), u[k], R(3));
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const R px = R(1) + eta[0][a], py = R(1) + eta[1][b];
+            const R xy = fma(g[0][a], py, g[1][b] * px);
+#pragma unroll
+            for (int c = 0; c < Lat<D>::NZ; ++c) {
+                if constexpr (D == 3) d[a + 3 * b + 9 * c] += fma(R(1) + eta[2][c], xy, g[2][c] * (px * py));
+                else d[a + 3 * b] += xy;
+            }
+        }
 }
 
 }  // namespace cm

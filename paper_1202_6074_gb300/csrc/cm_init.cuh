@@ -73,8 +73,7 @@ __global__ void __launch_bounds__(kBlock) k_init(S* __restrict__ dst, const type
     sfor<Q>([&](auto I) {
         constexpr int j = decltype(I)::value;
         constexpr int a = Lat<D>::ex(j) + 1, b = Lat<D>::ey(j) + 1, c = Lat<D>::ez(j) + 1;
-        constexpr R iw = (R)inv_weight<D>(j);
-        const R d = m[slot<D>(j)] * iw;
+        const R d = m[slot<D>(j)];
         const bool out = wx[a] || wy[b] || wz[c];
         if (out) {
             // the walls crossed going from x to x - e_j: e = +1 crosses the lower wall (side 0)
