@@ -98,16 +98,14 @@ template <int D, class S>
 cudaError_t launch_init(void* dst, const void* Ff, const Params& p, const double* rho, const double* u, cudaStream_t st,
                         int z0, int nzc) {
     using R = typename Codec<S>::R;
-    const dim3 b = cell_block(p.nx);
-    dim3 g = cell_grid(p, b);
-    g.z = nzc;
+    const auto l = cell_launch<R>(p, nzc, false);
     if constexpr (D == 3) {
         if (p.big) {
-            k_init<D, S, true><<<g, b, 0, st>>>((S*)dst, (const R*)Ff, typed<R>(p), rho, u, z0);
+            k_init<D, S, true><<<l.grid, l.block, 0, st>>>((S*)dst, (const R*)Ff, l.q, rho, u, z0);
             return cudaGetLastError();
         }
     }
-    k_init<D, S><<<g, b, 0, st>>>((S*)dst, (const R*)Ff, typed<R>(p), rho, u, z0);
+    k_init<D, S><<<l.grid, l.block, 0, st>>>((S*)dst, (const R*)Ff, l.q, rho, u, z0);
     return cudaGetLastError();
 }
 

@@ -22,15 +22,43 @@ constexpr int kBlock = 128;
 #endif
 constexpr long long kSmallGrid = CM_SMALL_GRID;
 template <class S> constexpr int step_min_blocks() { return sizeof(typename Codec<S>::R) == 8 ? 1 : CM_STEP_MIN_BLOCKS; }
+// blocks of rows: 128 threads a row, or fewer where that leaves a tenth fewer idle at its end (on D2Q9
+// 1500 x 701 FP32 blocks of 32 x 4, 2 % fewer threads, took 8 % longer)
+inline int padded_row(int nx, int bx) { return (nx + bx - 1) / bx * bx; }
 inline dim3 cell_block(int nx) {
-    int bx = 32;
-    while (bx < kBlock && bx < nx) bx *= 2;
+    int bx = kBlock;
+    for (int b = kBlock - 32; b >= 32; b -= 32)
+        if (10 * padded_row(nx, b) < 9 * padded_row(nx, bx)) bx = b;
     return dim3(bx, kBlock / bx, 1);
 }
 // the planes of a step launch: p.z0 .. p.z0 + step_planes(p) - 1
 inline int step_planes(const Params& p) { return p.nzc > 0 ? p.nzc : p.nz; }
 inline dim3 cell_grid(const Params& p, dim3 b) {
     return dim3((p.nx + b.x - 1) / b.x, (p.ny + b.y - 1) / b.y, step_planes(p));
+}
+// The launch of a one-cell-per-thread kernel over all planes of p: blocks of rows, or, where these
+// would leave a tenth of the threads idle or more, the rows end to end over the plane (plane_xy), for
+// the kernels that know that order: the FP64 step, which is bound by its arithmetic whether lanes are
+// idle or not, and the eddy-stress kernels. Against blocks of 32, 64 or 128 threads a row: FP64 runs
+// of 5 steps at 85^3 2533 -> 2214 us and at 130 x 96 x 96 5254 -> 4244 us, a filtered run at 130 x 97 x
+// 75 956 -> 889 us. The FP32 one-cell steps keep blocks of rows: finding the row by division made D2Q9
+// 1500 x 701 FP32 8 % slower even where it was not used.
+template <class R> struct CellLaunch {
+    PR<R> q;
+    dim3 block, grid;
+};
+template <class R> CellLaunch<R> cell_launch(const Params& p, int planes, bool flat, int threads = kBlock) {
+    CellLaunch<R> l{typed<R>(p), dim3(threads, 1, 1), dim3()};
+    const dim3 rows = threads == kBlock ? cell_block(p.nx) : l.block;
+    if (flat && p.nx > 1 && 10 * p.nx < 9 * padded_row(p.nx, rows.x)) {
+        set_flat(l.q, p.nx);
+        l.grid = dim3((unsigned)(((long long)p.nx * p.ny + threads - 1) / threads), 1, planes);
+    } else {
+        l.block = rows;
+        l.grid = cell_grid(p, l.block);
+        l.grid.z = planes;
+    }
+    return l;
 }
 
 // launch of a step kernel: with p.chain as a programmatic dependent of the kernel before it
@@ -80,16 +108,21 @@ __device__ __forceinline__ R smagorinsky_constant(const PR<R>& p, int y) {
 }
 
 // ---- fused pull + collide + store --------------------------------------------------------
-template <int D, class S, class FT>
+// FLAT: the rows laid end to end (plane_xy), for FP64
+template <int D, class S, class FT, bool FLAT = false>
 __global__ void __launch_bounds__(kBlock, step_min_blocks<S>()) k_step(const S* __restrict__ src, S* __restrict__ dst,
                                                 const typename Codec<S>::R* __restrict__ Ff, PR<typename Codec<S>::R> p) {
     using R = typename Codec<S>::R;
     constexpr int Q = Lat<D>::Q;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int x = blockIdx.x * blockDim.x + threadIdx.x;
+    int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = (int)blockIdx.z + p.z0;
     chain_begin();
-    if (x >= p.nx || y >= p.ny) return;
+    if constexpr (FLAT) {
+        if (!plane_xy(p, p.nx, x, y)) return;
+    } else {
+        if (x >= p.nx || y >= p.ny) return;
+    }
     chain_wait();
     using IX = Ix<FT::BIG>;
     const unsigned cell = (unsigned)((z * p.ny + y) * p.nx + x);
@@ -257,8 +290,14 @@ void launch_step_ft(const void* src, void* dst, const void* Ff, const Params& p,
     }
     // small grids: one warp per block so that the few blocks spread over as many SMs as possible
     // (the step is latency bound there; 128-thread blocks would leave most SMs idle)
-    const dim3 b = p.N <= kSmallGrid ? dim3(CM_SMALL_BLOCK, 1, 1) : cell_block(p.nx), g = cell_grid(p, b);
-    launch_chained(p, k_step<D, S, FT>, g, b, st, (const S*)src, (S*)dst, (const R*)Ff, typed<R>(p));
+    const auto l = cell_launch<R>(p, step_planes(p), sizeof(R) == 8, p.N <= kSmallGrid ? CM_SMALL_BLOCK : kBlock);
+    if constexpr (sizeof(R) == 8) {
+        if (l.q.flat_len) {
+            launch_chained(p, k_step<D, S, FT, true>, l.grid, l.block, st, (const S*)src, (S*)dst, (const R*)Ff, l.q);
+            return;
+        }
+    }
+    launch_chained(p, k_step<D, S, FT>, l.grid, l.block, st, (const S*)src, (S*)dst, (const R*)Ff, l.q);
 }
 
 // no force anywhere and unit rates above second order (the SIMPLE variant applies)
@@ -350,9 +389,9 @@ void launch_step_big_g(const void* src, void* dst, const void* Ff, const Params&
         }
         launch_pair<S, Feat<W, L, F, true, false, false, true>>(src, dst, Ff, p, st);
     } else {
-        const dim3 b = cell_block(p.nx), g = cell_grid(p, b);
-        launch_chained(p, k_step<3, S, Feat<W, L, F, true, false, false, true>>, g, b, st, (const S*)src, (S*)dst,
-                       (const R*)Ff, typed<R>(p));
+        const auto l = cell_launch<R>(p, step_planes(p), false);
+        launch_chained(p, k_step<3, S, Feat<W, L, F, true, false, false, true>>, l.grid, l.block, st, (const S*)src, (S*)dst,
+                       (const R*)Ff, l.q);
     }
 }
 template <class S>
@@ -413,20 +452,18 @@ template <int D, class S>
 cudaError_t launch_moments(const void* src, const void* Ff, const Params& p, double* rho, double* u, cudaStream_t st,
                            int z0, int nzc) {
     using R = typename Codec<S>::R;
-    const dim3 b = cell_block(p.nx);
-    dim3 g = cell_grid(p, b);
-    g.z = nzc;
+    const auto l = cell_launch<R>(p, nzc, false);
     if constexpr (D == 3) {
         if (p.big) {
-            if (has_walls(p)) k_moments<D, S, true, true><<<g, b, 0, st>>>((const S*)src, (const R*)Ff, typed<R>(p), rho, u, z0);
-            else k_moments<D, S, false, true><<<g, b, 0, st>>>((const S*)src, (const R*)Ff, typed<R>(p), rho, u, z0);
+            if (has_walls(p)) k_moments<D, S, true, true><<<l.grid, l.block, 0, st>>>((const S*)src, (const R*)Ff, l.q, rho, u, z0);
+            else k_moments<D, S, false, true><<<l.grid, l.block, 0, st>>>((const S*)src, (const R*)Ff, l.q, rho, u, z0);
             return cudaGetLastError();
         }
     }
     if (has_walls(p)) {
-        k_moments<D, S, true><<<g, b, 0, st>>>((const S*)src, (const R*)Ff, typed<R>(p), rho, u, z0);
+        k_moments<D, S, true><<<l.grid, l.block, 0, st>>>((const S*)src, (const R*)Ff, l.q, rho, u, z0);
     } else {
-        k_moments<D, S, false><<<g, b, 0, st>>>((const S*)src, (const R*)Ff, typed<R>(p), rho, u, z0);
+        k_moments<D, S, false><<<l.grid, l.block, 0, st>>>((const S*)src, (const R*)Ff, l.q, rho, u, z0);
     }
     return cudaGetLastError();
 }

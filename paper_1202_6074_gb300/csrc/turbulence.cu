@@ -18,10 +18,9 @@ template <int D, class S>
 __global__ void __launch_bounds__(kBlock) k_hydro_field(const S* __restrict__ src, const typename Codec<S>::R* __restrict__ Ff,
                                                        PR<typename Codec<S>::R> p, typename Codec<S>::R* __restrict__ q) {
     using R = typename Codec<S>::R;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int x, y;
     const int z = blockIdx.z;
-    if (x >= p.nx || y >= p.ny) return;
+    if (!plane_xy(p, p.nx, x, y)) return;
     const unsigned cell = (unsigned)((z * p.ny + y) * p.nx + x);
     R h[Lat<D>::Q];
     gather<D, S, false>(src, x, y, z, p, h);
@@ -50,10 +49,9 @@ __device__ __forceinline__ Nb neighbours(int x, int y, int z, const PR<R>& p) {
 // T = 2 C^2 |S| S with S_ij = (d_i u_j + d_j u_i) / 2; components xx, yy, zz, xy, xz, yz
 template <int D, class R>
 __global__ void __launch_bounds__(kBlock) k_eddy_stress(const R* __restrict__ q, PR<R> p, R cs2, R* __restrict__ T) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int x, y;
     const int z = blockIdx.z;
-    if (x >= p.nx || y >= p.ny) return;
+    if (!plane_xy(p, p.nx, x, y)) return;
     const unsigned N = p.N;
     const unsigned cell = (unsigned)((z * p.ny + y) * p.nx + x);
     const Nb nb = neighbours<R>(x, y, z, p);
@@ -81,10 +79,9 @@ __global__ void __launch_bounds__(kBlock) k_eddy_stress(const R* __restrict__ q,
 template <int D, class R>
 __global__ void __launch_bounds__(kBlock) k_turb_force(const R* __restrict__ q, const R* __restrict__ T, PR<R> p,
                                                       R* __restrict__ F) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int x, y;
     const int z = blockIdx.z;
-    if (x >= p.nx || y >= p.ny) return;
+    if (!plane_xy(p, p.nx, x, y)) return;
     const unsigned N = p.N;
     const unsigned cell = (unsigned)((z * p.ny + y) * p.nx + x);
     const Nb nb = neighbours<R>(x, y, z, p);
@@ -108,8 +105,9 @@ template <int D, class S>
 cudaError_t launch_turbulence_force(const void* state, void* force, const Params& p, double cs, void* scratch,
                                     cudaStream_t st) {
     using R = typename Codec<S>::R;
-    const dim3 b = cell_block(p.nx), g = cell_grid(p, b);
-    const PR<R> q = typed<R>(p);
+    const auto l = cell_launch<R>(p, p.nz, true);
+    const dim3 b = l.block, g = l.grid;
+    const PR<R>& q = l.q;
     R* hq = (R*)scratch;                 // [4][N] rho, u
     R* T = hq + 4 * (size_t)p.N;         // [6][N]
     k_hydro_field<D, S><<<g, b, 0, st>>>((const S*)state, (const R*)force, q, hq);

@@ -41,3 +41,20 @@ def test_one_step_elementwise(cm, name, storage, kernel):  # noqa: F811
     err = (got - ref).abs()
     assert bool((err <= ONE_STEP_ATOL[storage] + ONE_STEP_RTOL[storage] * ref.abs()).all()), f"{err.max().item():.3e}"
     s.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(33, 70), (57, 41), (130, 19), (129, 16), (1, 70)])
+@pytest.mark.parametrize("lattice", ["D2Q9", "D3Q27"])
+def test_fp64_rows_of_any_length(cm, lattice, nx, ny):  # noqa: F811
+    """The FP64 one-cell step lays rows that do not fill their blocks end to end over the plane."""
+    nz = 1 if lattice == "D2Q9" else 3
+    case = dict(lattice=lattice, shape=(nz, ny, nx), flow="tgv")
+    rho, u, F = _inputs(case)
+    s, o = _pair(cm, lattice, case["shape"], "f64", rho, u, F, tau=0.7, bc=("periodic", "bounceback", "periodic"))
+    o.set_state(H.decode(s.get_state(), lattice))
+    s.step(1)
+    o.step(1)
+    w = H.lattice(lattice).w.view(-1, 1, 1, 1)
+    err = (H.decode(s.get_state(), lattice) / w - o.s / w).abs().max().item()
+    assert err <= ONE_STEP_ATOL["f64"], f"{err:.3e}"
+    s.close()
