@@ -17,8 +17,8 @@ namespace cm {
 // Resident blocks per SM the register budget is sized for. The 16-bit steps are bound by
 // instruction latency rather than by HBM and gain from more resident warps where the registers
 // allow:
-//   6 blocks (at most 80 registers) for the unforced SIMPLE collision: +2 % over 5, while 7
-//     (72 registers, a 76-byte spill) lose 3 %;
+//   6 blocks (at most 80 registers) for the unforced SIMPLE collision: +1 % over 5, while 7
+//     (72 registers) lose 3 %;
 //   5 (at most 96) for the uniform force along x (FX): +1 % over 4, while 6 spill over 200 bytes;
 //   5 (at most 96) for the other forced steps without a force field (+5 % on the channel) and
 //     for the UNIT collision with a force field (+1.6 % on the isotropic turbulence LES; at 6
