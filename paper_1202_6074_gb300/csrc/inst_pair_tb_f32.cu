@@ -12,6 +12,10 @@ int two_steps_ft(const void* A, void* C, void* ring, const void* Ff, const Param
         if (simple_collision(p))
             return launch_pair_two_steps<float, Feat<W, L, false, false, true>>(A, C, ring, kTwoStepGroup,
                                                                                  kTwoStepRing, Ff, p, st);
+        // as single steps do, so that a pass gives their bits: a uniform force along x
+        if (p.F[1] == 0.0 && p.F[2] == 0.0 && p.omega3 == 1.0 && p.omega4 == 1.0)
+            return launch_pair_two_steps<float, Feat<W, L, false, false, false, true, false, true>>(
+                A, C, ring, kTwoStepGroup, kTwoStepRing, Ff, p, st);
     }
     return launch_pair_two_steps<float, Feat<W, L, F, false>>(A, C, ring, kTwoStepGroup, kTwoStepRing, Ff, p, st);
 }

@@ -41,3 +41,15 @@ def test_long_runs_equal_single_steps_bitwise(cm, name):  # noqa: F811
     assert a.launch_count - la == b.launch_count - lb
     a.close()
     b.close()
+
+
+def test_two_steps_per_pass_with_a_force_along_x(cm):  # noqa: F811
+    """The plane-ring schedule takes the collision variants of single steps: the same bits."""
+    rho, u, _ = _inputs(dict(lattice="D3Q27", shape=(18, 6, 64), flow="tgv_unforced"))
+    a, _ = _pair(cm, "D3Q27", (18, 6, 64), "f32", rho, u, uniform=(3e-4, 0.0, 0.0), kernel="pair_two_steps", tau=0.6)
+    b, _ = _pair(cm, "D3Q27", (18, 6, 64), "f32", rho, u, uniform=(3e-4, 0.0, 0.0), kernel="pair", tau=0.6)
+    a.step(5)
+    b.step(5)
+    assert torch.equal(a.get_state(), b.get_state())
+    a.close()
+    b.close()
