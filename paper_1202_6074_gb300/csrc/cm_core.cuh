@@ -111,8 +111,10 @@ template <class R> inline PR<R> typed(const Params& p) {
 // Chained launches: the steps captured into one graph follow each other as programmatic
 // dependents. A step's blocks are dispatched as soon as all blocks of the step before have
 // started and slots come free, work out their coordinates, and wait here until that step has
-// completed and its stores are visible; no global memory is read or written before the wait. A
-// kernel launched any other way passes both at once.
+// completed and its stores are visible; no global memory is read or written before the wait: the
+// populations are loaded by volatile statements with a memory clobber, which the wait orders
+// (ld_stream<true>, copy_async16). The force field may be read by .nc loads: no kernel of a chain writes it.
+// A kernel launched any other way passes both at once.
 __device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -312,64 +314,73 @@ __host__ __device__ constexpr double third_pow(int n) { return n == 0 ? 1.0 : n 
 // ------------------------------------------------------------------------------------------
 // Storage codec: d = fbar / w - 1 stored as S; arithmetic type R
 // ------------------------------------------------------------------------------------------
-// Read-only global loads with a 256-byte L2 prefetch hint: the pulled rows are streamed once,
+// Global loads of populations with a 256-byte L2 prefetch hint: the pulled rows are streamed once,
 // and fetching whole 256 B blocks measured 1.5 % faster for FP32 storage at 256^3 (no change
-// for 16-bit storage, which is issue bound).
-__device__ __forceinline__ double ld_stream(const double* p) {
+// for 16-bit storage, which is issue bound). CHAINED, for the kernels that may be launched chained:
+// the kernel before still writes these addresses while this one's blocks are already resident, so the
+// loads must neither go through the read-only path nor be moved above chain_wait(): coherent, volatile,
+// with a memory clobber. (The step kernels measured the same with either form, the adjoint step 3.5 %
+// slower with this one: the kernels that are never chained keep .nc.)
+template <bool CHAINED> __device__ __forceinline__ double ld_stream(const double* p) {
     double v;
-    asm("ld.global.nc.L2::256B.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    if constexpr (CHAINED) asm volatile("ld.global.L2::256B.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    else asm("ld.global.nc.L2::256B.f64 %0, [%1];" : "=d"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ float ld_stream(const float* p) {
+template <bool CHAINED> __device__ __forceinline__ float ld_stream(const float* p) {
     float v;
-    asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    if constexpr (CHAINED) asm volatile("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    else asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ unsigned short ld_stream(const unsigned short* p) {
+template <bool CHAINED> __device__ __forceinline__ unsigned short ld_stream(const unsigned short* p) {
     unsigned short v;
-    asm("ld.global.nc.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p));
+    if constexpr (CHAINED) asm volatile("ld.global.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+    else asm("ld.global.nc.L2::256B.b16 %0, [%1];" : "=h"(v) : "l"(p));
     return v;
 }
-
-__device__ __forceinline__ unsigned ld_stream(const unsigned* p) {
+template <bool CHAINED> __device__ __forceinline__ unsigned ld_stream(const unsigned* p) {
     unsigned v;
-    asm("ld.global.nc.L2::256B.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    if constexpr (CHAINED) asm volatile("ld.global.L2::256B.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    else asm("ld.global.nc.L2::256B.b32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ float2 ld_stream(const float2* p) {
+template <bool CHAINED> __device__ __forceinline__ float2 ld_stream(const float2* p) {
     float2 v;
-    asm("ld.global.nc.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    if constexpr (CHAINED) asm volatile("ld.global.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+    else asm("ld.global.nc.L2::256B.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
     return v;
 }
 
 // ld / st: one entry; ld2 / st2 (FP32 and 16-bit storage): the entries p[0], p[1] of two
-// adjacent cells in one access (p must be aligned to two entries), rounded as ld / st round
+// adjacent cells in one access (p must be aligned to two entries), rounded as ld / st round; CHAINED
+// as ld_stream
 template <class S> struct Codec;
 template <> struct Codec<double> {
     using R = double;
-    static __device__ __forceinline__ R ld(const double* p) { return ld_stream(p); }
+    template <bool CHAINED> static __device__ __forceinline__ R ld(const double* p) { return ld_stream<CHAINED>(p); }
     static __device__ __forceinline__ R ld_shared(const double* p) { return *p; }
     static __device__ __forceinline__ void st(double* p, R v) { *p = v; }
 };
 template <> struct Codec<float> {
     using R = float;
-    static __device__ __forceinline__ R ld(const float* p) { return ld_stream(p); }
+    template <bool CHAINED> static __device__ __forceinline__ R ld(const float* p) { return ld_stream<CHAINED>(p); }
     static __device__ __forceinline__ R ld_shared(const float* p) { return *p; }
     static __device__ __forceinline__ void st(float* p, R v) { *p = v; }
-    static __device__ __forceinline__ float2 ld2(const float* p) { return ld_stream(reinterpret_cast<const float2*>(p)); }
+    template <bool CHAINED> static __device__ __forceinline__ float2 ld2(const float* p) { return ld_stream<CHAINED>(reinterpret_cast<const float2*>(p)); }
     static __device__ __forceinline__ void st2(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
 };
 template <> struct Codec<__nv_bfloat16> {
     using R = float;
-    static __device__ __forceinline__ R ld(const __nv_bfloat16* p) {
-        return __bfloat162float(__ushort_as_bfloat16(ld_stream(reinterpret_cast<const unsigned short*>(p))));
+    template <bool CHAINED> static __device__ __forceinline__ R ld(const __nv_bfloat16* p) {
+        return __bfloat162float(__ushort_as_bfloat16(ld_stream<CHAINED>(reinterpret_cast<const unsigned short*>(p))));
     }
     static __device__ __forceinline__ R ld_shared(const __nv_bfloat16* p) {
         return __bfloat162float(__ushort_as_bfloat16(*reinterpret_cast<const unsigned short*>(p)));
     }
     static __device__ __forceinline__ void st(__nv_bfloat16* p, R v) { *p = __float2bfloat16_rn(v); }
-    static __device__ __forceinline__ float2 ld2(const __nv_bfloat16* p) {
-        const unsigned v = ld_stream(reinterpret_cast<const unsigned*>(p));   // BF16 = top half of an FP32
+    template <bool CHAINED> static __device__ __forceinline__ float2 ld2(const __nv_bfloat16* p) {
+        const unsigned v = ld_stream<CHAINED>(reinterpret_cast<const unsigned*>(p));   // BF16 = top half of an FP32
         return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
     }
     static __device__ __forceinline__ void st2(__nv_bfloat16* p, float a, float b) {
@@ -378,15 +389,15 @@ template <> struct Codec<__nv_bfloat16> {
 };
 template <> struct Codec<__half> {
     using R = float;
-    static __device__ __forceinline__ R ld(const __half* p) {
-        return __half2float(__ushort_as_half(ld_stream(reinterpret_cast<const unsigned short*>(p))));
+    template <bool CHAINED> static __device__ __forceinline__ R ld(const __half* p) {
+        return __half2float(__ushort_as_half(ld_stream<CHAINED>(reinterpret_cast<const unsigned short*>(p))));
     }
     static __device__ __forceinline__ R ld_shared(const __half* p) {
         return __half2float(__ushort_as_half(*reinterpret_cast<const unsigned short*>(p)));
     }
     static __device__ __forceinline__ void st(__half* p, R v) { *p = __float2half_rn(v); }
-    static __device__ __forceinline__ float2 ld2(const __half* p) {
-        const unsigned v = ld_stream(reinterpret_cast<const unsigned*>(p));
+    template <bool CHAINED> static __device__ __forceinline__ float2 ld2(const __half* p) {
+        const unsigned v = ld_stream<CHAINED>(reinterpret_cast<const unsigned*>(p));
         return __half22float2(*reinterpret_cast<const __half2*>(&v));
     }
     static __device__ __forceinline__ void st2(__half* p, float a, float b) {
@@ -462,6 +473,7 @@ template <int D, class S, bool WALLS, bool BIG = false, int PULL = kPullDev>
 __device__ __forceinline__ void gather_impl(const S* __restrict__ src, int x, int y, int z, const PR<typename Codec<S>::R>& p,
                                        typename Codec<S>::R (&h)[Lat<D>::Q]) {
     using R = typename Codec<S>::R;
+    constexpr bool CHAINED = PULL == kPullStored;      // the pull of k_step, which may run chained
     using IX = Ix<BIG>;
     // Q * S < 2^32 is checked at create for the 32-bit variant. On a slab, row offsets of the
     // ghost plane below are negative; they only occur for e_z = +1 (directions 18..26), so
@@ -509,7 +521,7 @@ __device__ __forceinline__ void gather_impl(const S* __restrict__ src, int x, in
             const bool bounced = bx || by || bz;
             const IX own = IX(Lat<D>::opp(i)) * PS + cell;
             const IX pulled = IX(i) * PS + row[c][b] + (unsigned)xs[a];
-            R d = Codec<S>::ld(src + (bounced ? own : pulled));
+            R d = Codec<S>::template ld<CHAINED>(src + (bounced ? own : pulled));
             if (p.moving) {
                 // half-way bounce-back from a moving wall: d += 6 (e . u_w), averaged over the
                 // walls the link crosses
@@ -522,7 +534,7 @@ __device__ __forceinline__ void gather_impl(const S* __restrict__ src, int x, in
             }
             h[slot<D>(i)] = PULL == kPullStored ? d : PULL == kPullDev ? d * w : fma(d, w, w);
         } else {
-            const R d = Codec<S>::ld(src + (IX(i) * PS + row[c][b] + (unsigned)xs[a]));
+            const R d = Codec<S>::template ld<CHAINED>(src + (IX(i) * PS + row[c][b] + (unsigned)xs[a]));
             h[slot<D>(i)] = PULL == kPullStored ? d : PULL == kPullDev ? d * w : fma(d, w, w);
         }
     });

@@ -161,15 +161,15 @@ __device__ __forceinline__ void gather_pair(const S* __restrict__ src, int x, in
             const bool by = WALLS && yo[b], bz = WALLS && zo[c];
             const bool bA = a == 2 && xoA, bB = a == 0 && xoB;      // the links across the x walls
             const IX own = IX(Lat<3>::opp(i)) * PS;
-            float da = Codec<S>::ld(src + (by || bz || bA ? own + cellA : base + (unsigned)xa[a]));
-            float db = Codec<S>::ld(src + (by || bz || bB ? own + cellB : base + (unsigned)xb[a]));
+            float da = Codec<S>::template ld<true>(src + (by || bz || bA ? own + cellA : base + (unsigned)xa[a]));
+            float db = Codec<S>::template ld<true>(src + (by || bz || bB ? own + cellB : base + (unsigned)xb[a]));
             if (p.moving) add_wall_motion<i>(p, by, bz, bA, bB, da, db);
             h[slot<3>(i)] = F2(da, db);
         } else {
             if constexpr (sizeof(S) == 2)   // 64-bit row pointers (measured faster at 16-bit storage)
-                h[slot<3>(i)] = F2(Codec<S>::ld(src + xa[a] + base), Codec<S>::ld(src + xb[a] + base));
+                h[slot<3>(i)] = F2(Codec<S>::template ld<true>(src + xa[a] + base), Codec<S>::template ld<true>(src + xb[a] + base));
             else
-                h[slot<3>(i)] = F2(Codec<S>::ld(src + (base + (unsigned)xa[a])), Codec<S>::ld(src + (base + (unsigned)xb[a])));
+                h[slot<3>(i)] = F2(Codec<S>::template ld<true>(src + (base + (unsigned)xa[a])), Codec<S>::template ld<true>(src + (base + (unsigned)xb[a])));
         }
     });
 }
@@ -218,18 +218,18 @@ __device__ __forceinline__ void gather_adj(const S* __restrict__ src, int x0, in
             const IX back = IX(Lat<3>::opp(i)) * PS + own;       // the cells' own reflected entries
             float2 d;
             if constexpr (a == 1) {
-                d = Codec<S>::ld2(src + (by || bz ? back : base + (unsigned)x0));
+                d = Codec<S>::template ld2<true>(src + (by || bz ? back : base + (unsigned)x0));
             } else {
-                d.x = Codec<S>::ld(src + (by || bz || bA ? back : base + (unsigned)c0[a]));
-                d.y = Codec<S>::ld(src + (by || bz || bB ? back + 1u : base + (unsigned)c1[a]));
+                d.x = Codec<S>::template ld<true>(src + (by || bz || bA ? back : base + (unsigned)c0[a]));
+                d.y = Codec<S>::template ld<true>(src + (by || bz || bB ? back + 1u : base + (unsigned)c1[a]));
             }
             if (p.moving) add_wall_motion<i>(p, by, bz, bA, bB, d.x, d.y);
             h[slot<3>(i)] = F2(d.x, d.y);
         } else if constexpr (a == 1) {
-            const float2 d = Codec<S>::ld2(src + x0 + base);
+            const float2 d = Codec<S>::template ld2<true>(src + x0 + base);
             h[slot<3>(i)] = F2(d.x, d.y);
         } else {
-            h[slot<3>(i)] = F2(Codec<S>::ld(src + c0[a] + base), Codec<S>::ld(src + c1[a] + base));
+            h[slot<3>(i)] = F2(Codec<S>::template ld<true>(src + c0[a] + base), Codec<S>::template ld<true>(src + c1[a] + base));
         }
     });
 }
@@ -260,12 +260,12 @@ __device__ __forceinline__ void gather_adj_inner(const S* __restrict__ src, int 
         constexpr int a = Lat<3>::ex(i) + 1, b = Lat<3>::ey(i) + 1, c = Lat<3>::ez(i) + 1;
         const S* __restrict__ q = px + (IX(i) * PS + (unsigned)((zs[c] * p.ny + ys[b]) * p.nx));
         if constexpr (a == 1) {
-            const float2 d = Codec<S>::ld2(q);
+            const float2 d = Codec<S>::template ld2<true>(q);
             h[slot<3>(i)] = F2(d.x, d.y);
         } else if constexpr (a == 0) {          // e_x = -1: columns x0 + 1, x0 + 2
-            h[slot<3>(i)] = F2(Codec<S>::ld(q + 1), Codec<S>::ld(q + 2));
+            h[slot<3>(i)] = F2(Codec<S>::template ld<true>(q + 1), Codec<S>::template ld<true>(q + 2));
         } else {                                // e_x = +1: columns x0 - 1, x0
-            h[slot<3>(i)] = F2(Codec<S>::ld(q - 1), Codec<S>::ld(q));
+            h[slot<3>(i)] = F2(Codec<S>::template ld<true>(q - 1), Codec<S>::template ld<true>(q));
         }
     });
 }

@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(TX + 32, 2) k_step_tma(const __grid_constant__
                         if (ox) { const int sd = ex > 0 ? 0 : 1; wx += p.uw[0][sd][0]; wy += p.uw[0][sd][1]; wz += p.uw[0][sd][2]; cnt += 1; }
                         if (oy) { const int sd = ey > 0 ? 0 : 1; wx += p.uw[1][sd][0]; wy += p.uw[1][sd][1]; wz += p.uw[1][sd][2]; cnt += 1; }
                         if (oz) { const int sd = ez > 0 ? 0 : 1; wx += p.uw[2][sd][0]; wy += p.uw[2][sd][1]; wz += p.uw[2][sd][2]; cnt += 1; }
-                        d = Codec<S>::ld(src + (Lat<3>::opp(i) * N + cell)) +
+                        d = Codec<S>::template ld<false>(src + (Lat<3>::opp(i) * N + cell)) +
                             R(6) * (R(ex) * wx + R(ey) * wy + R(ez) * wz) / cnt;
                     }
                 }
