@@ -842,6 +842,18 @@ __device__ __forceinline__ R shear_rate(const R (&P)[6], R irho, const PR<scalar
 // the first-order central moment it is: M += K_x, and 3 K / rho beside 3 u in eta of y and z before
 // their one rounding. Without it the error of an FP32 run against 64 bits grew by a third
 // (Couette 1500 x 701, 100 steps); 16-bit storage rounds a thousand times coarser.
+// FINE (FP32 storage): where one velocity component is small, the e = 0 term -3/2 u^2 of its axis is
+// below the last place of what the other axes leave, and adding it to a value that is already
+// rounded drops it every time, while the e = +-1 terms 3 u^2 +- 3 u are rounded to either side: mass
+// grew by up to 5e-11 a cell and step (u_z of 1e-5 beside 0.02; Taylor-Green 128^3, 60 steps: 9e-10
+// in all, 3e-12 with the transforms, -2e-11 now). So rho phi_z - 1 is kept as a sum of two values, exact but
+// for the rounding of rho eta_z, whose low part enters before the last sum E = high + (low + ...),
+// and E is added to the sum of the small terms of E' and t2, not to each of them. No bias is
+// left that 6e6 random cells would show (below 1e-12 a cell and step in twelve mixes of small and
+// large components), and the errors of FP32 runs are at or below the transforms' (mean of 15
+// flows at 32^3, 90 steps: unforced 6.99e-7 against 7.26e-7, with a force along x 1.35e-5 against
+// 1.58e-5). About 40 operations a cell, on steps that wait for HBM. FP64 has the same effect at u of 1e-9,
+// 16-bit storage rounds the populations 1e4 times coarser than the bias: they do without.
 // Everything stays a deviation from the rest state. About 310 operations a cell (350 with the force)
 // instead of the 416 (540) of the two transforms (D3Q27), which the 16-bit steps and FP64 are bound
 // by. Measured, against the transforms, per step: Taylor-Green 256^3 BF16 316 -> 304 us, D2Q9 1500 x
@@ -855,7 +867,7 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
     static_assert(product_form<FT>(), "the product form is the Maxwellian one at unit rates");
     constexpr int NZ = Lat<D>::NZ;
     const R C = R((T)moment_scale<D>());
-    const R third = R(T(1) / 3);
+    constexpr bool FINE = COMP && std::is_same_v<T, float>;
     raw_x<D, R>(m);
     // sums over the lines of one e_z with the weights (1, 4, 1) of e_y: raw moments of order
     // (x, y) = 00 (A), 01 (Y), 02 (Q), 10 (B), 11 (W), 20 (X)
@@ -874,7 +886,7 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
         if constexpr (D == 3) return fma(R(4), v[1], v[0] + v[2]);
         else return v[0];
     };
-    const R drho = over_z(A) * C, Rx = over_z(B) * C, jy = over_z(Y) * C;
+    const R mass = over_z(A), drho = mass * C, Rx = over_z(B) * C, jy = over_z(Y) * C;
     const R rho = R(1) + drho, irho = rcp(rho);
     const R cd = drho * R(T(-1) / 3);
     R jx = Rx, Rm = Rx;                  // j_x = R_x + F / 2, R_x - F / 2
@@ -940,14 +952,15 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
         s21 = f * R(0.5);
         s22 = Fh;
     }
-    auto x_line = [&](int l, R E, R Ep, R M, R S) {
+    auto x_line = [&](int l, R E, R Ep, R M, R S) {       // S without E if FINE
         if constexpr (FT::FX) {
             M = fma(s11, m[3 * l], M);
             S = fma(s22, m[3 * l + 1], fma(s21, m[3 * l], S + s20));
         }
         const R V = Ep + R(1);
         const R r1 = fma(ux, V, M);
-        const R t2 = fma(qx3, V, fma(x6, M, S));
+        R t2 = fma(qx3, V, fma(x6, M, S));
+        if constexpr (FINE) t2 = E + t2;
         m[3 * l] = fma(R(-3), r1, t2);
         m[3 * l + 1] = fma(R(-0.5), t2, Ep * R(1.5));
         m[3 * l + 2] = fma(R(3), r1, t2);
@@ -961,22 +974,47 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
         R ez[3], z0[3], z1[3];
         tables(uz, jz, ez, z0, z1);
         const R zz[3] = {Tzz * R(3), Tzz * R(-1.5), Tzz * R(3)};   // T_zz g_2(z)
+        // FINE: rho phi_z - 1 = zh + zl (the two-sum of rho eta_z and the unrounded drho), rho phi_z
+        R zh[3], zl[3], rz[3];
+        if constexpr (FINE) {
+            const R dl = fma(mass, C, -drho);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const R v = rho * ez[c];
+                zh[c] = fma(rho, ez[c], drho);
+                const R t = zh[c] - v;
+                zl[c] = ((v - (zh[c] - t)) + (drho - t)) + dl;
+                rz[c] = R(1) + zh[c];
+            }
+        }
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
             const R phi = R(1) + ey[b], yz1 = Tyz * y1[b], xy1 = Txy * y1[b], xx0 = Txx3 * y0[b], xz0 = Txz * y0[b];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const R E = fma(rho, fma(phi, ez[c], ey[b]), drho);
-                const R Ep = fma(yy[b], z0[c], fma(y0[b], zz[c], fma(yz1, z1[c], E)));
-                const R M = fma(xy1, z0[c], M0 ? fma(xz0, z1[c], m0) : xz0 * z1[c]);
-                x_line(3 * c + b, E, Ep, M, fma(xx0, z0[c], E));
+                if constexpr (FINE) {
+                    const R E = zh[c] + fma(rz[c], ey[b], zl[c]);
+                    const R Ep = E + fma(yy[b], z0[c], fma(y0[b], zz[c], yz1 * z1[c]));
+                    const R M = fma(xy1, z0[c], fma(xz0, z1[c], m0));
+                    x_line(3 * c + b, E, Ep, M, xx0 * z0[c]);
+                } else {
+                    const R E = fma(rho, fma(phi, ez[c], ey[b]), drho);
+                    const R Ep = fma(yy[b], z0[c], fma(y0[b], zz[c], fma(yz1, z1[c], E)));
+                    const R M = fma(xy1, z0[c], M0 ? fma(xz0, z1[c], m0) : xz0 * z1[c]);
+                    x_line(3 * c + b, E, Ep, M, fma(xx0, z0[c], E));
+                }
             }
         }
     } else {
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const R E = fma(rho, ey[b], drho);
-            x_line(b, E, E + yy[b], M0 ? fma(Txy, y1[b], m0) : Txy * y1[b], fma(Txx3, y0[b], E));
+            if constexpr (FINE) {       // the e_y = 0 term onto the unrounded drho
+                const R E = b == 1 ? fma(mass, C, rho * ey[b]) : fma(rho, ey[b], drho);
+                x_line(b, E, E + yy[b], fma(Txy, y1[b], m0), Txx3 * y0[b]);
+            } else {
+                const R E = fma(rho, ey[b], drho);
+                x_line(b, E, E + yy[b], M0 ? fma(Txy, y1[b], m0) : Txy * y1[b], fma(Txx3, y0[b], E));
+            }
         }
     }
 }
