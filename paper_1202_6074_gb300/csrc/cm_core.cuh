@@ -837,11 +837,14 @@ __device__ __forceinline__ R shear_rate(const R (&P)[6], R irho, const PR<scalar
 // Evaluated line by line along x: with E = rho phi_y phi_z - 1, E' = E + its T part of x order 0,
 // M = the T part and source of order 1, S = E + 3 x those of order 2 and V = 1 + E':
 //   r1 = u V + M,  t2 = 3 u^2 V + 6 u M + S,  d_+- = t2 +- 3 r1,  d_0 = 3/2 E' - t2 / 2
-// COMP (FP32 storage): u = j / rho is rounded, and rho u then misses the momentum by the same
+// COMP (FP32 and FP64 storage): u = j / rho is rounded, and rho u then misses the momentum by the same
 // relative error in every direction at once. The residual K = j - rho u (exact, one fma) goes in as
-// the first-order central moment it is: M += K_x, and 3 K / rho beside 3 u in eta of y and z before
-// their one rounding. Without it the error of an FP32 run against 64 bits grew by a third
-// (Couette 1500 x 701, 100 steps); 16-bit storage rounds a thousand times coarser.
+// the first-order central moment it is: M += K_x, and 3 K (for 3 K / rho) beside 3 u in eta before its
+// one rounding, or, along y in FP64, where operations count, the momentum 3 j_y itself in the place
+// of 3 rho u_y. Without it the error of an FP32 run against 64 bits grew by a third (Couette 1500 x
+// 701, 100 steps), and an FP64 step rounded a cell's momentum 12 % (D3Q27) to 20 % (D2Q9) worse than the
+// transforms; with it FP64 is 4 % better to equal, at 1.6 % of the D2Q9 step's time and nothing at D3Q27
+// 128^3. 16-bit storage rounds a thousand times coarser and does without.
 // FINE (FP32 storage): where one velocity component is small, the e = 0 term -3/2 u^2 of its axis is
 // below the last place of what the other axes leave, and adding it to a value that is already
 // rounded drops it every time, while the e = +-1 terms 3 u^2 +- 3 u are rounded to either side: mass
@@ -917,13 +920,15 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
     const R Txy = omn * P[3], Txz = omn * P[4], Tyz = omn * P[5];
 
     // 1D populations over the 1D weights, index e + 1
-    auto tables = [&](R u, R j, R (&eta)[3], R (&g0)[3], R (&g1)[3]) {
-        const R q = u * u, q3 = q * R(3);
-        R lo = q3, hi = q3;
-        if constexpr (COMP) {
-            const R k = fma(-rho, u, j) * (irho * R(3));
-            lo = q3 - k;
-            hi = q3 + k;
+    auto tables = [&](auto RES, R u, R j, R (&eta)[3], R (&g0)[3], R (&g1)[3]) {     // RES: with 3 K
+        const R q = u * u;
+        R lo, hi;
+        if constexpr (decltype(RES)::value) {
+            const R k = fma(-rho, u, j) * R(3);
+            lo = fma(R(3), q, -k);
+            hi = fma(R(3), q, k);
+        } else {
+            lo = hi = q * R(3);
         }
         eta[1] = q * R(-1.5);
         eta[0] = fma(R(-3), u, lo);
@@ -936,7 +941,15 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
         g1[2] = fma(R(6), u, R(3));
     };
     R ey[3], y0[3], y1[3];
-    tables(uy, jy, ey, y0, y1);
+    tables(std::bool_constant<FINE>{}, uy, jy, ey, y0, y1);
+    // FP64: rho phi_y - 1 with the momentum 3 j_y itself in the place of 3 rho u_y
+    R G[3];
+    if constexpr (COMP && !FINE) {
+        const R g = fma(rho, uy * uy * R(3), drho);
+        G[0] = fma(R(-3), jy, g);
+        G[1] = fma(rho, ey[1], drho);
+        G[2] = fma(R(3), jy, g);
+    }
     const R x6 = ux * R(6), qx3 = ux * ux * R(3);
     R Kx = R(0);
     if constexpr (COMP) Kx = fma(-rho, ux, jx);
@@ -972,7 +985,7 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
     const R yy[3] = {Tyy * R(3), Tyy * R(-1.5), Tyy * R(3)};       // T_yy g_2(y)
     if constexpr (D == 3) {
         R ez[3], z0[3], z1[3];
-        tables(uz, jz, ez, z0, z1);
+        tables(std::bool_constant<COMP>{}, uz, jz, ez, z0, z1);
         const R zz[3] = {Tzz * R(3), Tzz * R(-1.5), Tzz * R(3)};   // T_zz g_2(z)
         // FINE: rho phi_z - 1 = zh + zl (the two-sum of rho eta_z and the unrounded drho), rho phi_z
         R zh[3], zl[3], rz[3];
@@ -989,6 +1002,8 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
         }
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
+            R rphi;
+            if constexpr (COMP && !FINE) rphi = R(1) + G[b];
             const R phi = R(1) + ey[b], yz1 = Tyz * y1[b], xy1 = Txy * y1[b], xx0 = Txx3 * y0[b], xz0 = Txz * y0[b];
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
@@ -998,7 +1013,7 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
                     const R M = fma(xy1, z0[c], fma(xz0, z1[c], m0));
                     x_line(3 * c + b, E, Ep, M, xx0 * z0[c]);
                 } else {
-                    const R E = fma(rho, fma(phi, ez[c], ey[b]), drho);
+                    const R E = COMP ? fma(rphi, ez[c], G[b]) : fma(rho, fma(phi, ez[c], ey[b]), drho);
                     const R Ep = fma(yy[b], z0[c], fma(y0[b], zz[c], fma(yz1, z1[c], E)));
                     const R M = fma(xy1, z0[c], M0 ? fma(xz0, z1[c], m0) : xz0 * z1[c]);
                     x_line(3 * c + b, E, Ep, M, fma(xx0, z0[c], E));
@@ -1012,7 +1027,7 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
                 const R E = b == 1 ? fma(mass, C, rho * ey[b]) : fma(rho, ey[b], drho);
                 x_line(b, E, E + yy[b], fma(Txy, y1[b], m0), Txx3 * y0[b]);
             } else {
-                const R E = fma(rho, ey[b], drho);
+                const R E = COMP ? G[b] : fma(rho, ey[b], drho);
                 x_line(b, E, E + yy[b], M0 ? fma(Txy, y1[b], m0) : Txy * y1[b], fma(Txx3, y0[b], E));
             }
         }

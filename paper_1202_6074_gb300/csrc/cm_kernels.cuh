@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kBlock, step_min_blocks<S>()) k_step(const S* 
     R F[3];
     load_force<R, FT::FIELD, FT::BIG>(Ff, p, cell, F);
     // the collision returns the stored deviations (inverse weights folded into its last sweep)
-    collide<D, R, FT, true, sizeof(S) == 4>(h, F, p, smagorinsky_constant<R, FT::LES>(p, y));
+    collide<D, R, FT, true, (sizeof(S) >= 4)>(h, F, p, smagorinsky_constant<R, FT::LES>(p, y));
     sfor<Q>([&](auto I) {
         constexpr int i = decltype(I)::value;
         Codec<S>::st(dst + (IX(i) * PS + cell), h[slot<D>(i)]);

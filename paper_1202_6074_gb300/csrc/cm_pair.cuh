@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kBlock, pair_min_blocks<S, FT>()) k_step_pair(
         for (int d = 0; d < 3; ++d) F[d] = F2(p.F[d]);
     }
     constexpr bool DEV = pair_dev<S, FT>();
-    collide<3, F2, FT, DEV, sizeof(S) == 4>(h, F, p, smagorinsky_constant<float, FT::LES>(p, y));
+    collide<3, F2, FT, DEV, (sizeof(S) >= 4)>(h, F, p, smagorinsky_constant<float, FT::LES>(p, y));
     sfor<27>([&](auto I) {
         constexpr int i = decltype(I)::value;
         const F2 v = DEV ? h[slot<3>(i)] : h[slot<3>(i)] * F2((float)inv_weight_scaled<3>(i));
