@@ -40,7 +40,12 @@ inline bool pair_eligible(const Params& p, int D, bool fp32_arith) {
 }
 // The same kernel on any row length, and with x walls: what the automatic choice takes for the
 // other D3Q27 grids with FP32 arithmetic. The line is drawn on the plane (a slab of a grid takes
-// the same kernel as the whole grid, so that their results stay equal bit for bit).
+// the same kernel as the whole grid, so that their results stay equal bit for bit). One cell against two
+// cells per thread, us a step: 24^3 FP32 1.9 / 2.9, BF16 1.9 / 2.5; 32^3 2.6 / 3.2, 2.6 / 2.5; 40^3 4.4 /
+// 4.1, 4.4 / 3.7; 48 x 48 x 16 3.0 / 3.1, 3.0 / 2.6; 48^3 4.7 / 4.5, 5.1 / 3.7; 100 x 100 x 60 22.0 /
+// 19.0, 17.5 / 11.5. With walls across x, where one cell per thread diverges, two are faster at
+// all of these sizes (24^3 4.8 / 4.2, 40^3 9.8 / 5.4). So the line lies where most flows gain; on flat
+// boxes just above it (48 x 48 x 8, 90 x 70 x 4) an unforced step loses up to 0.7 us.
 constexpr int kRaggedPairPlane = 2048;
 inline bool ragged_pair_eligible(const Params& p, int D, bool fp32_arith) {
     return D == 3 && fp32_arith && !p.big && p.nx >= 8 && (long long)p.nx * p.ny >= kRaggedPairPlane;

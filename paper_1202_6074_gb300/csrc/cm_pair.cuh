@@ -51,7 +51,9 @@ constexpr int pair_min_blocks() {
 // of two entries (e_x = +-1 populations stay two single-entry reads), which removes a third of
 // the memory instructions and half of the address arithmetic. Measured on the 256^3 steps:
 // +12 % (Taylor-Green) and +14 % (forced LES) at 16-bit storage, +3 % for the forced FP32 LES,
-// but -1 % for the unforced FP32 step, which stays on (x, x + nx/2).
+// but -1 % for the unforced FP32 step, which stays on (x, x + nx/2) where rows are a multiple of 64
+// cells. On other even rows the second half starts off the 32-byte sectors that a warp's accesses
+// fill, and adjacent cells are faster there too (launch_pair_ragged).
 template <class S, class FT> constexpr bool pair_adjacent() { return sizeof(S) == 2 || !FT::SIMPLE; }
 
 // Whether the collision returns the stored deviations with the inverse weights folded into its
@@ -417,7 +419,10 @@ void launch_pair(const void* src, void* dst, const void* Ff, const Params& p, cu
     launch_chained(p, k_step_pair<S, FT>, g, b, st, (const S*)src, (S*)dst, (const float*)Ff, typed<float>(p), planes);
 }
 
-// The same on rows of any length (Params::pair == 2). Adjacent cells also need even rows.
+// The same on rows of any length (Params::pair == 2). Adjacent cells also need even rows. They are taken
+// in every variant: unforced FP32, (x, x + nx/2) against adjacent cells, us a step: 60^3 7.30 / 6.31,
+// 96^3 29.9 / 29.6, 120^3 59.2 / 55.8, 200 x 200 x 100 136.1 / 126.9, a cavity 130 x 111 x 90 54.8 / 51.9
+// (one cell per thread: 6.43, 30.2, 56.3, 132.5, 66.2).
 template <class S, class FT>
 void launch_pair_ragged(const void* src, void* dst, const void* Ff, const Params& p, cudaStream_t st) {
     const int half = (p.nx + 1) / 2;
@@ -426,7 +431,7 @@ void launch_pair_ragged(const void* src, void* dst, const void* Ff, const Params
     const dim3 g((unsigned)(((long long)half * p.ny + kBlock - 1) / kBlock), 1, step_planes(p));
     Ring planes{};
     planes.z0 = p.z0;
-    if constexpr (pair_adjacent<S, FT>()) {
+    {
         const uintptr_t two = 2 * sizeof(S);
         if (p.nx % 2 == 0 && (uintptr_t)src % two == 0 && (uintptr_t)dst % two == 0) {
             launch_chained(p, k_step_pair<S, FT, false, false, true, true>, g, kBlock, st, (const S*)src, (S*)dst,
