@@ -170,7 +170,10 @@ CMLBM_API int cmlbm_set_stream(cmlbm_t* h, void* stream);
 
 /* Set the body force (paper: F in Eqs. cascadedLBE1 - velocitycalculation). uniform[3] is
  * added to every cell; field (FP64, [3][N], on `where`) replaces it when non-NULL and is
- * copied into the handle in the arithmetic precision (FP64 or FP32). NULL uniform = 0. */
+ * copied into the handle in the arithmetic precision (FP64 or FP32). NULL uniform = 0.
+ * A uniform force along x alone has a shorter form of the collision (omega_3 = omega_4 = 1, standard
+ * attractor and compressibility): it agrees with the same force given as a field to rounding, not
+ * to the bit. */
 CMLBM_API int cmlbm_set_force(cmlbm_t* h, const double uniform[3], const double* field, int where);
 
 /* Initialise the state so that the next pull returns fbar = f^M(rho, u) - S/2 with the
