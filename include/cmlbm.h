@@ -186,11 +186,11 @@ CMLBM_API int cmlbm_init(cmlbm_t* h, const double* rho, const double* u, int whe
 
 /* Advance nsteps stream-and-collide steps (nsteps >= 0): the pull of Eq. cascadedstreaming1
  * followed by the collision of Sec. 10, fused in one kernel launch per step, asynchronous on the
- * handle's stream. Pairs of steps, and on grids of up to 2,000,000 cells sixteen steps where a
+ * handle's stream. Pairs of steps, and sixteen steps where the state is at most 256 MiB and a
  * call asks for thirty-two or more, are replayed as a CUDA graph (captured once per buffer parity
  * on a private stream, dropped when the force changes), so a call of many steps costs one graph
- * launch per two or sixteen steps; a failed capture falls back to plain launches for the handle's
- * life. */
+ * launch per two or sixteen steps. A capture that failed is not tried again in the handle's life:
+ * sixteen steps fall back to pairs, pairs to plain launches. */
 CMLBM_API int cmlbm_step(cmlbm_t* h, int nsteps);
 
 /* One step from the state buffer src into dst (device pointers of cmlbm_state_bytes() each,

@@ -63,6 +63,7 @@ struct cmlbm {
     cudaStream_t cap = nullptr;
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     cudaGraphExec_t glong[2] = {nullptr, nullptr};     // kLongGraph steps (single steps only)
+    bool long_graphs = true;                           // no capture of kLongGraph steps has failed
     // two steps per pass: the plane ring of the intermediate state (allocated on first use)
     bool two_steps = false;
     void* ring = nullptr;
@@ -223,16 +224,19 @@ void drop_graphs(cmlbm* h) {
     }
 }
 
-// Steps per graph launch where steps are short: every graph launch costs the stream a gap, which the
-// steps inside one graph do not have between them. Measured (runs of 100, 500 and 100 steps, graphs
-// of 2 -> graphs of 16): D3Q27 32^3 FP32 422 -> 287 us, D2Q9 64 x 32 FP64 4114 -> 3344 us, D2Q9
-// 1500 x 701 FP32 1264 -> 1110 us. Graphs of 8 are up to 6 % slower on steps of 5 us and more, graphs
-// of 48 take 3.7 us a step at 32^3 where graphs of 16 take 2.7. The chaining alone is worth 2 to 6 %
-// (a step at 64^3: FP32 7.30 -> 7.07 us, BF16 6.41 -> 6.02 us; nothing at 32^3). Above kLongGraphCells
-// a step takes 50 us or more and the gap is lost in it; the graph of two then spares the capture
-// of sixteen.
+// Steps per graph launch: every graph launch costs the stream a gap, which the steps inside one graph
+// do not have between them. Graphs of sixteen instead of two steps take 1.4 to 1.8 us off every step,
+// whatever its size (us a step, graphs of 2 / 16: D2Q9 1500 x 701 FP32 11.3 / 9.9, 2000 x 1200 FP32 27.7 /
+// 26.3, 3000 x 2000 BF16 52.1 / 50.4; D3Q27 32^3 FP32 4.2 / 2.7, 128^3 BF16 40.8 / 39.2, 128^3 FP32 68.5 /
+// 67.0, 256^3 FP32 517.0 / 515.6). Graphs of 8 are up to 6 % slower on steps of 5 us and more, graphs of 48
+// take 3.7 us a step at 32^3 where graphs of 16 take 2.7. The limit is on the bytes of a state, since the
+// time of a step goes with them: 256 MB take 75 us or more to read and write, and beyond that the gap
+// is below 2 % and the graph of two spares the capture of sixteen.
+// A call has to ask for thirty-two steps before sixteen are captured. A caller who changes the force
+// before every call pays the capture each time; set_force and step(n), graphs of 16 / 2, us: D3Q27 32^3
+// FP32 n = 32: 159 / 155, 48: 209 / 223, 96: 359 / 422; 64^3 BF16 32: 263 / 284; D2Q9 64 x 32 FP64 32: 221 / 224.
 constexpr int kLongGraph = 16;
-constexpr long long kLongGraphCells = 2000000;
+constexpr size_t kLongGraphBytes = (size_t)256 << 20;
 
 // Enqueue two steps from buf[k]: buf[k] -> buf[1-k] -> buf[k] as two single steps, or, on a
 // two-steps handle, one pass buf[k] -> buf[1-k] through the plane ring (the state then ends in
@@ -650,13 +654,14 @@ int cmlbm_step(cmlbm_t* h, int nsteps) {
     }
     // pairs of steps as graph replays (one graph launch instead of two or more kernel launches)
     if (nsteps >= 2 && h->graphs && !h->tma) {
-        // sixteen steps a graph where steps are short and a call asks for enough of them
+        // sixteen steps a graph where steps are short and a call asks for enough of them (kLongGraphBytes)
         const int cur = h->cur;
-        if (!h->two_steps && h->p.N <= kLongGraphCells && nsteps >= kLongGraph) {
+        if (!h->two_steps && h->long_graphs && cmlbm_state_bytes(h) <= kLongGraphBytes && nsteps >= kLongGraph) {
             if (!h->glong[cur] && nsteps >= 2 * kLongGraph &&
                 capture_steps(h, cur, kLongGraph, &h->glong[cur]) != cudaSuccess) {
                 cudaGetLastError();
                 h->glong[cur] = nullptr;
+                h->long_graphs = false;      // for the handle's life: graphs of two, or plain launches
             }
             for (; nsteps >= kLongGraph && h->glong[cur]; nsteps -= kLongGraph) {
                 cudaError_t e = cudaGraphLaunch(h->glong[cur], h->st);

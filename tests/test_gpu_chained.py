@@ -2,8 +2,8 @@
 steps launched one by one: the same kernels in the same order, so the same bits.
 
 The staged 16-bit step is taken where every resident warp has 8 tiles of 64 cells or more (60 with a
-force field); the grids here have a quarter more than that on this device's multiprocessors. Grids of up
-to 2,000,000 cells run graphs of sixteen steps, larger ones graphs of two.
+force field); the grids here have a quarter more than that on this device's multiprocessors. States of
+up to 256 MiB run graphs of sixteen steps, larger ones graphs of two.
 """
 import pytest
 import torch
@@ -16,10 +16,10 @@ CHANNEL = dict(bc=("periodic", "bounceback", "periodic"), smagorinsky_cs=0.1, va
 # rows (nx, ny), tiles per resident warp and resident warps per multiprocessor behind the planes
 CASES = {
     "staged_unforced": dict(row=(128, 128), tiles=8 * 20, kw=dict(omega_bulk=1.0)),
-    "staged_unforced_walls_graphs_of_two": dict(row=(192, 133), tiles=16 * 20,
+    "staged_unforced_walls_graphs_of_two": dict(row=(192, 133), tiles=24 * 20,
                                                 kw=dict(bc=("periodic", "bounceback", "bounceback"), smagorinsky_cs=0.1)),
     "staged_channel": dict(row=(192, 61), tiles=8 * 16, force="x", kw=CHANNEL),
-    "staged_channel_graphs_of_two": dict(row=(256, 101), tiles=16 * 16, force="x", kw=CHANNEL),
+    "staged_channel_graphs_of_two": dict(row=(256, 101), tiles=30 * 16, force="x", kw=CHANNEL),
     "staged_field": dict(row=(256, 256), tiles=60 * 16, force="field", kw=dict(smagorinsky_cs=0.1, omega_bulk=1.0)),
     "two_cells_x_force": dict(shape=(9, 20, 128), force="x", kw=dict(omega_bulk=1.0)),
     "ragged_x_force": dict(shape=(5, 33, 66), force="x", kw=dict(bc=("bounceback", "bounceback", "periodic"))),
@@ -39,8 +39,10 @@ def _shape(case, margin=1.25):
     return (int(margin * case["tiles"] * sms / (nx // 64 * ny)) + 1, ny, nx)
 
 
-def _compare(cm, lattice, shape, storage, case):  # noqa: F811
+def _compare(cm, lattice, shape, storage, name, case):  # noqa: F811
     nz, ny, nx = shape
+    if "row" in case:
+        assert (27 * 2 * nx * ny * nz > 256 << 20) == ("graphs_of_two" in name or "field" in name)
     g = torch.Generator(device="cuda").manual_seed(11)
     kw = dict(dict(tau=0.53), **case["kw"])
     a, b = (cm.Solver(lattice=lattice, nx=nx, ny=ny, nz=nz, storage=storage, **kw) for _ in range(2))
@@ -68,10 +70,10 @@ def _compare(cm, lattice, shape, storage, case):  # noqa: F811
 @pytest.mark.parametrize("storage", ["bf16", "f16"])
 @pytest.mark.parametrize("name", list(CASES))
 def test_chained_16_bit_steps_equal_single_steps_bitwise(cm, name, storage):  # noqa: F811
-    _compare(cm, "D3Q27", _shape(CASES[name]), storage, CASES[name])
+    _compare(cm, "D3Q27", _shape(CASES[name]), storage, name, CASES[name])
 
 
 @pytest.mark.parametrize("name", list(PLAIN))
 def test_chained_steps_equal_single_steps_bitwise(cm, name):  # noqa: F811
     case = PLAIN[name]
-    _compare(cm, case["lattice"], case["shape"], case["storage"], case)
+    _compare(cm, case["lattice"], case["shape"], case["storage"], name, case)
