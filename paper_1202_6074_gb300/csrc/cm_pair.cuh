@@ -378,16 +378,21 @@ __global__ void __launch_bounds__(kBlock, pair_min_blocks<S, FT>()) k_step_pair(
 }
 
 // k_step_async (cm_async.cuh) takes the 16-bit steps in product form and those with a force field on
-// grids that give every resident warp eight tiles of 64 cells or more (sixty with a force field);
-// below that a warp has too few tiles to copy ahead in. Unforced BF16, us a step, k_step_pair
-// against k_step_async: 64^3 5.3 / 6.5, 128 x 96 x 64 13.2 / 16.1, 128 x 128 x 96 30.6 / 30.2, 192^3
-// 132 / 121; a force along x: 128 x 96 x 96 28.0 / 26.8; a force field: 192 x 160 x 128 97.2 / 99.3,
-// 256 x 192 x 192 226.4 / 225.2, 512^3 3180 / 3100. src must be aligned to its 16-byte copies. The lane
-// arithmetic is the same: so are the bits.
+// grids that give every resident warp enough tiles of 64 cells to copy ahead in (async_tiles): 8 unforced,
+// 7 with a force along x, 60 with a force field. BF16, us a step, k_step_pair against k_step_async, by
+// tiles (on 152 multiprocessors the lines lie at 24,320, 17,024 and 145,920):
+//   unforced: 12,288 13.1 / 15.9; 18,432 22.2 / 22.3; 24,576 30.3 / 30.0 (walls, eddy viscosity 31.4 /
+//     32.1); 27,648 34.4 / 33.8 (35.6 / 35.4); 110,592 131 / 120
+//   force along x: 12,288 15.9 / 18.2; 15,360 20.7 / 20.1 (channel 22.1 / 22.3); 16,896 23.7 / 22.2 (25.0 /
+//     24.5); 18,432 26.3 / 24.7 (28.0 / 27.1); 24,576 34.5 / 31.7; 110,592 147 / 125
+//   force field: 61,440 95.2 / 96.8; 110,592 167.5 / 166.9; 147,456 220.4 / 220.3; 262,144 388 / 385;
+//     512^3 3180 / 3100
+// src must be aligned to its 16-byte copies. The lane arithmetic is the same: so are the bits.
 template <class S, class FT> constexpr bool async_variant() {
     return sizeof(S) == 2 && (product_form<FT>() || (FT::FIELD && FT::UNIT && !FT::GEN));
 }
 template <class FT> __host__ __device__ constexpr int async_blocks();
+template <class FT> constexpr int async_tiles() { return FT::FIELD ? 60 : FT::FX ? 7 : 8; }
 template <class FT> inline int async_resident_warps(const Params& p) { return p.nsm * async_blocks<FT>() * (kBlock / 32); }
 template <class S, class FT>
 void launch_async(const void* src, void* dst, const void* Ff, const Params& p, cudaStream_t st);
@@ -401,7 +406,7 @@ void launch_pair(const void* src, void* dst, const void* Ff, const Params& p, cu
     planes.z0 = p.z0;
     if constexpr (async_variant<S, FT>()) {
         const long long tiles = (long long)(p.nx / 64) * p.ny * step_planes(p);
-        if (tiles >= (FT::FIELD ? 60 : 8) * async_resident_warps<FT>(p) && (uintptr_t)src % 16 == 0 && (uintptr_t)dst % 4 == 0) {
+        if (tiles >= async_tiles<FT>() * async_resident_warps<FT>(p) && (uintptr_t)src % 16 == 0 && (uintptr_t)dst % 4 == 0) {
             launch_async<S, FT>(src, dst, Ff, p, st);
             return;
         }
