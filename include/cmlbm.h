@@ -70,6 +70,8 @@ enum { CMLBM_DEVICE = 0, CMLBM_HOST = 1 };                         /* where a bu
 enum { CMLBM_ATTRACTOR_MAXWELL = 0, CMLBM_ATTRACTOR_FACTORIZED = 1 };
 enum { CMLBM_KERNEL_AUTO = 0, CMLBM_KERNEL_DIRECT = 1, CMLBM_KERNEL_TMA = 2, CMLBM_KERNEL_PAIR = 3,
        CMLBM_KERNEL_PAIR_TWO_STEPS = 4 };
+enum { CMLBM_PATH_NONE = 0, CMLBM_PATH_ONE_CELL = 1, CMLBM_PATH_TWO_CELLS = 2, CMLBM_PATH_RAGGED = 3,
+       CMLBM_PATH_STAGED = 4, CMLBM_PATH_TWO_STEPS = 5, CMLBM_PATH_TMA = 6 };
 
 typedef struct cmlbm cmlbm_t;
 
@@ -343,9 +345,17 @@ CMLBM_API long long cmlbm_launch_count(const cmlbm_t* h);
 /* The step kernel the handle runs: CMLBM_KERNEL_DIRECT, CMLBM_KERNEL_PAIR,
  * CMLBM_KERNEL_PAIR_TWO_STEPS or CMLBM_KERNEL_TMA (what CMLBM_KERNEL_AUTO resolved to, as a
  * value that an explicit request of the same configuration accepts: on grids that PAIR does not
- * cover, AUTO answers CMLBM_KERNEL_DIRECT whichever of the two it runs there);
+ * cover, AUTO answers CMLBM_KERNEL_DIRECT whichever of the two it runs there: see
+ * cmlbm_step_path);
  * CMLBM_ERR_INVALID for a NULL handle. */
 CMLBM_API int cmlbm_step_kernel(const cmlbm_t* h);
+
+/* The kernel that the handle's last step (cmlbm_step, cmlbm_step_buffers, cmlbm_step_split or
+ * cmlbm_step_filtered) was launched with, or last captured with where steps are replayed as graphs:
+ * one cell per thread, two cells per thread on whole-warp rows or on rows of any length, the
+ * 16-bit step with its pull staged ahead in shared memory, two steps per pass, or the TMA-staged
+ * step. CMLBM_PATH_NONE before the first step; CMLBM_ERR_INVALID for a NULL handle. */
+CMLBM_API int cmlbm_step_path(const cmlbm_t* h);
 
 /* ---- allocation-free reduction (no counterpart in the paper) --------------------------- *
  * The FP64 reductions of cmlbm_reduce for callers that cannot allocate device memory: a host

@@ -31,7 +31,8 @@ SYMBOLS = ["cmlbm_config_default", "cmlbm_create", "cmlbm_destroy", "cmlbm_last_
            "cmlbm_moments_of", "cmlbm_reduce", "cmlbm_state_bytes", "cmlbm_get_state", "cmlbm_set_state",
            "cmlbm_adjoint_terminal", "cmlbm_step_adjoint", "cmlbm_launch_count", "cmlbm_reduce_noalloc",
            "cmlbm_turbulence_force", "cmlbm_step_filtered", "cmlbm_halo_bytes", "cmlbm_halo_pack",
-           "cmlbm_halo_unpack", "cmlbm_step_kernel", "cmlbm_step_adjoint_segment", "cmlbm_step_split"]
+           "cmlbm_halo_unpack", "cmlbm_step_kernel", "cmlbm_step_adjoint_segment", "cmlbm_step_split", "cmlbm_step_path"]
+PATHS = {0: None, 1: "one_cell", 2: "two_cells", 3: "ragged", 4: "staged", 5: "two_steps", 6: "tma"}
 KERNELS = {0: "auto", 1: "direct", 2: "tma", 3: "pair", 4: "pair_two_steps"}
 
 
@@ -104,6 +105,7 @@ def load():
         "cmlbm_halo_pack": (I, [P, I, P, I]),
         "cmlbm_halo_unpack": (I, [P, I, P, I]),
         "cmlbm_step_kernel": (I, [P]),
+        "cmlbm_step_path": (I, [P]),
     }
     for name, (res, args) in sig.items():
         fn = getattr(lib, name)
@@ -220,6 +222,12 @@ class Solver:
     def step_kernel(self):
         """"direct", "pair" or "tma": the step kernel this handle runs."""
         return KERNELS[int(self.lib.cmlbm_step_kernel(self.h))]
+
+    @property
+    def step_path(self):
+        """The kernel of the last step launched or captured: "one_cell", "two_cells", "ragged", "staged",
+        "two_steps" or "tma"; None before the first step."""
+        return PATHS[int(self.lib.cmlbm_step_path(self.h))]
 
     # ---- API --------------------------------------------------------------------------
     def set_force(self, uniform=(0.0, 0.0, 0.0), field=None):

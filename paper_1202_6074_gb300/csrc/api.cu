@@ -68,6 +68,7 @@ struct cmlbm {
     bool two_steps = false;
     void* ring = nullptr;
     int pass_launches = 0;     // kernel launches of one two-step pass
+    int path = cm::kPathNone;  // kernel of the last step launched or captured (cmlbm_step_path)
 #ifdef CM_NO_GRAPHS
     bool graphs = false;       // build option: plain launches only
 #else
@@ -169,6 +170,7 @@ cudaError_t dispatch(const cmlbm* h, Fn&& fn) {
 
 // TMA-staged step when the handle has maps for src (one of its buffers, or maps made here).
 cudaError_t do_step_tma(cmlbm* h, const void* map_main, const void* map_halo, const void* src, void* dst) {
+    h->path = cm::kPathTma;
     switch (h->cfg.storage) {
         case CMLBM_F32: return cm::launch_step_tma<float>(map_main, map_halo, src, dst, h->force, h->p, h->flag, h->nsm, h->st);
         case CMLBM_BF16: return cm::launch_step_tma<__nv_bfloat16>(map_main, map_halo, src, dst, h->force, h->p, h->flag, h->nsm, h->st);
@@ -244,6 +246,7 @@ constexpr size_t kLongGraphBytes = (size_t)256 << 20;
 cudaError_t enqueue_two_steps(cmlbm* h, int k) {
     if (h->two_steps) {
         const int n = cm::launch_two_steps_f32(h->buf[k], h->buf[1 - k], h->ring, h->force, h->p, h->st);
+        h->path = cm::kPathTwoSteps;
         if (n < 0) return cudaErrorInvalidValue;
         h->pass_launches = n;
         h->launches += n;
@@ -387,6 +390,7 @@ int cmlbm_create(const cmlbm_config* cfg, cmlbm_t** out) {
     h->st = (cudaStream_t)c.stream;
     cm::Params& p = h->p;
     std::memset(&p, 0, sizeof(p));
+    p.path = &h->path;
     p.nx = c.nx;
     p.ny = c.ny;
     p.nz = c.nz;
@@ -531,6 +535,12 @@ int cmlbm_step_kernel(const cmlbm_t* h) {
     if (h->two_steps) return CMLBM_KERNEL_PAIR_TWO_STEPS;
     return h->p.pair == 1 ? CMLBM_KERNEL_PAIR : CMLBM_KERNEL_DIRECT;
 }
+
+static_assert(cm::kPathOneCell == CMLBM_PATH_ONE_CELL && cm::kPathTwoCells == CMLBM_PATH_TWO_CELLS &&
+                  cm::kPathRagged == CMLBM_PATH_RAGGED && cm::kPathStaged == CMLBM_PATH_STAGED &&
+                  cm::kPathTwoSteps == CMLBM_PATH_TWO_STEPS && cm::kPathTma == CMLBM_PATH_TMA,
+              "cmlbm_step_path returns the recorded values");
+int cmlbm_step_path(const cmlbm_t* h) { return h ? h->path : CMLBM_ERR_INVALID; }
 
 size_t cmlbm_state_bytes(const cmlbm_t* h) { return h ? (size_t)h->Q * (size_t)h->p.S * h->esize : 0; }
 

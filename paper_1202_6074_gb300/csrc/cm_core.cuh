@@ -48,6 +48,7 @@ struct Params {
     int nsm;               // multiprocessors of the device
     int big;               // Q * S >= 2^32: kernels with 64-bit element offsets
     int chain;             // launch as a dependent of the kernel before it (chain_wait)
+    int* path;             // where a step launch records its kernel (kPath...; NULL: nowhere)
     int z0, nzc;           // planes z0 .. z0 + nzc - 1 of a step launch (nzc = 0: all planes)
     long long N;           // cells updated (nx ny nz)
     long long S;           // elements between direction planes of a state buffer (N, or nx ny (nz + 2) on a slab)
@@ -81,6 +82,12 @@ template <class R> struct PR {
     R tau0, omega_bulk, omega3, omega4, cs, vd_aplus, vd_utau_nu, rho0;
     R omega_nu;            // 1 / tau0, IEEE-rounded on the host (used by the FP64 collision)
 };
+
+// the step kernels that a launch records in Params::path (the values of cmlbm_step_path)
+enum { kPathNone = 0, kPathOneCell = 1, kPathTwoCells = 2, kPathRagged = 3, kPathStaged = 4, kPathTwoSteps = 5, kPathTma = 6 };
+inline void record_path(const Params& p, int path) {
+    if (p.path) *p.path = path;
+}
 
 template <class R> inline PR<R> typed(const Params& p) {
     PR<R> q;

@@ -288,6 +288,7 @@ void launch_step_ft(const void* src, void* dst, const void* Ff, const Params& p,
             return;
         }
     }
+    record_path(p, kPathOneCell);
     // small grids: one warp per block so that the few blocks spread over as many SMs as possible
     // (the step is latency bound there; 128-thread blocks would leave most SMs idle)
     const auto l = cell_launch<R>(p, step_planes(p), sizeof(R) == 8, p.N <= kSmallGrid ? CM_SMALL_BLOCK : kBlock);
@@ -386,6 +387,7 @@ void launch_step_big_g(const void* src, void* dst, const void* Ff, const Params&
         }
         launch_pair<S, Feat<W, L, F, true, false, false, true>>(src, dst, Ff, p, st);
     } else {
+        record_path(p, kPathOneCell);
         const auto l = cell_launch<R>(p, step_planes(p), false);
         launch_chained(p, k_step<3, S, Feat<W, L, F, true, false, false, true>>, l.grid, l.block, st, (const S*)src, (S*)dst,
                        (const R*)Ff, l.q);

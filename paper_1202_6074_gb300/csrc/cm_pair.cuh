@@ -407,10 +407,12 @@ void launch_pair(const void* src, void* dst, const void* Ff, const Params& p, cu
     if constexpr (async_variant<S, FT>()) {
         const long long tiles = (long long)(p.nx / 64) * p.ny * step_planes(p);
         if (tiles >= async_tiles<FT>() * async_resident_warps<FT>(p) && (uintptr_t)src % 16 == 0 && (uintptr_t)dst % 4 == 0) {
+            record_path(p, kPathStaged);
             launch_async<S, FT>(src, dst, Ff, p, st);
             return;
         }
     }
+    record_path(p, kPathTwoCells);
     // adjacent cells need both buffers aligned to two entries (buffers passed in by the caller
     // may be offset); the force field is the library's own allocation
     if constexpr (pair_adjacent<S, FT>()) {
@@ -433,6 +435,7 @@ void launch_pair_ragged(const void* src, void* dst, const void* Ff, const Params
     const int half = (p.nx + 1) / 2;
     PR<float> q = typed<float>(p);
     set_flat(q, half);
+    record_path(p, kPathRagged);
     const dim3 g((unsigned)(((long long)half * p.ny + kBlock - 1) / kBlock), 1, step_planes(p));
     Ring planes{};
     planes.z0 = p.z0;
