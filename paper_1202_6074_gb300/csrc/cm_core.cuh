@@ -47,7 +47,7 @@ struct Params {
                            // (periodic x, nx a multiple of 64), 2 = any row length, x walls included
     int nsm;               // multiprocessors of the device
     int big;               // Q * S >= 2^32: kernels with 64-bit element offsets
-    int chain;             // launch as a dependent of the kernel before it (chain_wait)
+    int chain;             // launch as a dependent of the kernel before it, where that pays (chain_pays)
     int* path;             // where a step launch records its kernel (kPath...; NULL: nowhere)
     int z0, nzc;           // planes z0 .. z0 + nzc - 1 of a step launch (nzc = 0: all planes)
     long long N;           // cells updated (nx ny nz)

@@ -61,6 +61,24 @@ template <class R> CellLaunch<R> cell_launch(const Params& p, int planes, bool f
     return l;
 }
 
+// Whether a chained launch of this many blocks pays. Its blocks are dispatched to whatever slots the step
+// before leaves first. Up to two blocks a multiprocessor, and from one full wave on, that only saves
+// the gap between the steps; in between the blocks that come first pile up on the multiprocessors that
+// are done first, and the step takes as long as the fullest of them. Graphs of sixteen, us a step, not
+// chained / chained: 16 x 32 x 16 FP32 2.2 / 1.9, D2Q9 83 x 69 FP64 5.4 / 5.0, 64^3 BF16 5.5 / 5.1, 96^3
+// BF16 16.9 / 16.6, 128^3 FP32 67.1 / 66.9; in between D2Q9 196 x 168 FP64 9.0 / 14.0, D2Q9 256 x 256 FP64
+// 16.9 / 24.7, 24^3 FP64 12.4 / 20.0, a cavity 64 x 16 x 84 FP32 7.7 / 9.8, 48 x 18 x 47 FP32 with a
+// force field 3.3 / 4.6 (and with fewer operations also 48 x 16 x 32 FP32 2.4 / 2.2, 64 x 64 x 48 FP16
+// 5.0 / 4.6, which are given up).
+template <class K> bool chain_pays(const Params& p, K kernel, dim3 grid, dim3 block, int smem) {
+    const long long blocks = (long long)grid.x * grid.y * grid.z;
+    if (blocks <= 2LL * p.nsm) return true;
+    int resident = 0;
+    const int threads = (int)(block.x * block.y * block.z);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, threads, (size_t)smem) != cudaSuccess) return false;
+    return blocks >= (long long)resident * p.nsm;
+}
+
 // launch of a step kernel: with p.chain as a programmatic dependent of the kernel before it
 template <class... P, class... A>
 inline void launch_chained_smem(const Params& p, void (*kernel)(P...), dim3 grid, dim3 block, int smem, cudaStream_t st,
@@ -74,7 +92,7 @@ inline void launch_chained_smem(const Params& p, void (*kernel)(P...), dim3 grid
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     c.attrs = &at;
-    c.numAttrs = p.chain ? 1 : 0;
+    c.numAttrs = p.chain && chain_pays(p, kernel, grid, block, smem) ? 1 : 0;
     cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 template <class... P, class... A>
