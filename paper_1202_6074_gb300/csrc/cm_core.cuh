@@ -1049,13 +1049,13 @@ __device__ __forceinline__ void collide_product(R (&m)[Lat<D>::Q], R Fx, const P
 // sweep); otherwise the deviation populations h, each scaled by 2^n (n = |e_x| + |e_y| + |e_z|
 // of its direction, see central_inverse_impl), which the caller stores as h * inv_weight_scaled.
 // R is the arithmetic type (double, float, or F2 for two cells of one row; cs_eff and the
-// parameters are then scalars shared by both cells).
+// parameters are then scalars shared by both cells). PRODUCT: in product form (collide_product).
 // ------------------------------------------------------------------------------------------
-template <int D, class R, class FT, bool DEV = false, bool COMP = false>
+template <int D, class R, class FT, bool DEV = false, bool COMP = false, bool PRODUCT = product_form<FT>()>
 __device__ __forceinline__ void collide(R (&m)[Lat<D>::Q], const R F[3], const PR<scalar_t<R>>& p, scalar_t<R> cs_eff) {
     using T = scalar_t<R>;
     constexpr int Q = Lat<D>::Q;
-    if constexpr (product_form<FT>()) {
+    if constexpr (PRODUCT) {
         static_assert(DEV, "the product form returns the deviations");
         collide_product<D, R, FT, COMP>(m, F[0], p, cs_eff);
         return;
