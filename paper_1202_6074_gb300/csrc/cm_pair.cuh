@@ -436,18 +436,25 @@ void launch_pair_ragged(const void* src, void* dst, const void* Ff, const Params
     PR<float> q = typed<float>(p);
     set_flat(q, half);
     record_path(p, kPathRagged);
-    const dim3 g((unsigned)(((long long)half * p.ny + kBlock - 1) / kBlock), 1, step_planes(p));
+    // Blocks of one warp where blocks of four would not fill the multiprocessors once: they spread more
+    // evenly. Graphs of sixteen, us a step, blocks of 128 / 32 threads: 60 x 60 x 32 FP32 4.6 / 4.2, FP16
+    // with a force field 5.6 / 4.9; 46 x 46 x 24 FP32 4.0 / 3.3; 48 x 48 x 8 FP32 2.6 / 2.3; a cavity 60 x 60 x
+    // 32 FP32 5.8 / 5.3; 90 x 70 x 4 BF16 2.5 / 2.7. Above one wave they lose up to 12 % (120^3 FP32).
+    const long long pairs = (long long)half * p.ny;
+    const bool few = (pairs + kBlock - 1) / kBlock * step_planes(p) <= (long long)p.nsm * pair_min_blocks<S, FT>();
+    const int b = few ? 32 : kBlock;
+    const dim3 g((unsigned)((pairs + b - 1) / b), 1, step_planes(p));
     Ring planes{};
     planes.z0 = p.z0;
     {
         const uintptr_t two = 2 * sizeof(S);
         if (p.nx % 2 == 0 && (uintptr_t)src % two == 0 && (uintptr_t)dst % two == 0) {
-            launch_chained(p, k_step_pair<S, FT, false, false, true, true>, g, kBlock, st, (const S*)src, (S*)dst,
+            launch_chained(p, k_step_pair<S, FT, false, false, true, true>, g, b, st, (const S*)src, (S*)dst,
                            (const float*)Ff, q, planes);
             return;
         }
     }
-    launch_chained(p, k_step_pair<S, FT, false, false, false, true>, g, kBlock, st, (const S*)src, (S*)dst,
+    launch_chained(p, k_step_pair<S, FT, false, false, false, true>, g, b, st, (const S*)src, (S*)dst,
                    (const float*)Ff, q, planes);
 }
 

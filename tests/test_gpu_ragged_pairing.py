@@ -3,6 +3,7 @@ entries: every cell goes through the same lane arithmetic either way, so the bit
 import pytest
 import torch
 
+from paper_1202_6074_gb300 import slab as SL
 from test_gpu_parity import cm  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -43,3 +44,31 @@ def test_pairings_agree_bitwise(cm, name, storage):  # noqa: F811
     assert torch.isfinite(outs[0].float()).all()
     assert torch.equal(outs[0].view(torch.uint8), outs[1].view(torch.uint8))
     s.close()
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("nx", [66, 67])
+def test_block_sizes_agree_bitwise(cm, nx, storage):  # noqa: F811
+    """A grid whose blocks of 128 threads fill the multiprocessors more than once, against four slabs
+    of it, which run blocks of one warp."""
+    ny, sms = 32, torch.cuda.get_device_properties(0).multi_processor_count
+    planes = (nx + 1) // 2 * ny // 128 + 1
+    nz = 7 * sms // planes + 2                 # up to six blocks a multiprocessor are one wave
+    g = torch.Generator(device="cuda").manual_seed(6)
+    u = 0.03 * torch.randn((3, nz, ny, nx), generator=g, device="cuda", dtype=torch.float64)
+    kw = dict(lattice="D3Q27", nx=nx, ny=ny, storage=storage, tau=0.53)
+    whole = cm.Solver(nz=nz, **kw)
+    whole.init(None, u)
+    parts = 4
+    slabs = []
+    for r in range(parts):
+        s, z0 = SL.cuda_slab(cm, nz, r, parts, **kw)
+        s.init(None, u[:, z0:z0 + s.shape[0]].contiguous())
+        slabs.append(s)
+    SL.SlabRun(slabs, SL.LocalExchange(slabs)).step(3)
+    whole.step(3)
+    assert whole.step_path == slabs[0].step_path == "ragged"
+    own = torch.cat([s.get_state()[:, 1:-1] for s in slabs], dim=1)
+    assert torch.equal(own.view(torch.uint8), whole.get_state().view(torch.uint8))
+    for s in slabs + [whole]:
+        s.close()
