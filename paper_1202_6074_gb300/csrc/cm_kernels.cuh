@@ -23,12 +23,15 @@ constexpr int kBlock = 128;
 constexpr long long kSmallGrid = CM_SMALL_GRID;
 template <class S> constexpr int step_min_blocks() { return sizeof(typename Codec<S>::R) == 8 ? 1 : CM_STEP_MIN_BLOCKS; }
 // blocks of rows: 128 threads a row, or fewer where that leaves a tenth fewer idle at its end (on D2Q9
-// 1500 x 701 FP32 blocks of 32 x 4, 2 % fewer threads, took 8 % longer)
+// 1500 x 701 FP32 blocks of 32 x 4, 2 % fewer threads, took 8 % longer). fp64: without blocks of 96 threads,
+// whose three warps leave one of a multiprocessor's four FP64 pipes idle: FP64 with a force field, us a step
+// with 96 x 1 / 32 x 4 threads: 94 x 64 x 24 189.0 / 168.5, 95 x 64 x 64 441.9 /
+// 440.3
 inline int padded_row(int nx, int bx) { return (nx + bx - 1) / bx * bx; }
-inline dim3 cell_block(int nx) {
+inline dim3 cell_block(int nx, bool fp64 = false) {
     int bx = kBlock;
     for (int b = kBlock - 32; b >= 32; b -= 32)
-        if (10 * padded_row(nx, b) < 9 * padded_row(nx, bx)) bx = b;
+        if (!(fp64 && kBlock % b != 0) && 10 * padded_row(nx, b) < 9 * padded_row(nx, bx)) bx = b;
     return dim3(bx, kBlock / bx, 1);
 }
 // the planes of a step launch: p.z0 .. p.z0 + step_planes(p) - 1
@@ -49,7 +52,7 @@ template <class R> struct CellLaunch {
 };
 template <class R> CellLaunch<R> cell_launch(const Params& p, int planes, bool flat, int threads = kBlock) {
     CellLaunch<R> l{typed<R>(p), dim3(threads, 1, 1), dim3()};
-    const dim3 rows = threads == kBlock ? cell_block(p.nx) : l.block;
+    const dim3 rows = threads == kBlock ? cell_block(p.nx, sizeof(R) == 8) : l.block;
     if (flat && p.nx > 1 && 10 * p.nx < 9 * padded_row(p.nx, rows.x)) {
         set_flat(l.q, p.nx);
         l.grid = dim3((unsigned)(((long long)p.nx * p.ny + threads - 1) / threads), 1, planes);

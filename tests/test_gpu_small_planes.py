@@ -21,6 +21,9 @@ CASES = {
     "d3q27_tiny": dict(lattice="D3Q27", shape=(2, 3, 4), kw=dict(tau=0.6)),
     "d3q27_walls_les": dict(lattice="D3Q27", shape=(5, 9, 33), kw=dict(tau=0.53, smagorinsky_cs=0.15, van_driest=(26.0, 8.0), wall_velocity=WALL,
                                                                        bc=("bounceback", "bounceback", "periodic"))),
+    # above 65,536 cells: blocks of several rows, of which the plane's last are partly empty
+    "d2q9_rows_of_94": dict(lattice="D2Q9", shape=(1, 702, 94), kw=dict(tau=0.6)),
+    "d3q27_rows_of_94_walls": dict(lattice="D3Q27", shape=(38, 19, 94), kw=dict(tau=0.56, bc=("periodic", "bounceback", "periodic"), wall_velocity=WALL)),
     "d3q27_rows_of_7": dict(lattice="D3Q27", shape=(4, 40, 7), kw=dict(tau=0.56, omega_bulk=1.0)),
 }
 
