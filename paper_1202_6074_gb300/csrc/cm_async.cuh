@@ -8,7 +8,7 @@
 // beside them that the e_x = +-1 rows are read into: 26 copies of 16 bytes, one instruction of the
 // warp. The collision then reads its populations at constant offsets from one shared-memory
 // address, without the address arithmetic of 45 global loads (warp instructions per 32 cells of the
-// unforced step: 400 -> 359).
+// unforced step: 400 -> 366).
 // Measured per step against k_step_pair (same collision): Taylor-Green 256^3 BF16 304 -> 275 us
 // (6.6 TB/s of 108 B a cell), channel LES 1024 x 256 x 256 BF16 1430 -> 1250 us, force-field LES 512^3 BF16
 // 3180 -> 3100 us. A copy ahead into L2 instead (cp.async.bulk.prefetch) was 15 % slower: what is

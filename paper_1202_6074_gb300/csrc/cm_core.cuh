@@ -116,12 +116,12 @@ template <class R> inline PR<R> typed(const Params& p) {
 }
 
 // Chained launches: the steps captured into one graph follow each other as programmatic
-// dependents. A step's blocks are dispatched as soon as all blocks of the step before have
-// started and slots come free, work out their coordinates, and wait here until that step has
-// completed and its stores are visible; no global memory is read or written before the wait: the
-// populations are loaded by volatile statements with a memory clobber, which the wait orders
-// (ld_stream<true>, copy_async16). The force field may be read by .nc loads: no kernel of a chain writes it.
-// A kernel launched any other way passes both at once.
+// dependents, where that pays (chain_pays). A step's blocks are dispatched as soon as all blocks of
+// the step before have started and slots come free, work out their coordinates, and wait here until
+// that step has completed and its stores are visible; no global memory is read or written before the
+// wait: the populations are loaded by volatile statements with a memory clobber, which the wait orders
+// (ld_stream<true>, copy_async16). The force field may be read by .nc loads: no kernel of a chain writes
+// it. A kernel launched any other way passes both at once.
 __device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

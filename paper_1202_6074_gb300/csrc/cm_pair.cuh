@@ -275,7 +275,7 @@ __device__ __forceinline__ void gather_adj_inner(const S* __restrict__ src, int 
 // RAG: rows of any length (laid end to end over the blocks, plane_xy) and walls across x. A
 // variant of its own: the few instructions more cost the 16-bit steps of whole-warp rows 2.5 %.
 // Against the one-cell kernel, which these grids ran before (per step of a 50-step run): a cavity
-// 130 x 111 x 90 FP32 79.6 -> 56.7 us, the factorized attractor 150 x 97 x 75 FP16 47.3 -> 35.1 us.
+// 130 x 111 x 90 FP32 79.6 -> 51.9 us, the factorized attractor 150 x 97 x 75 FP16 47.3 -> 33.5 us.
 template <class S, class FT, bool RS = false, bool RD = false, bool ADJ = false, bool RAG = false>
 __global__ void __launch_bounds__(kBlock, pair_min_blocks<S, FT>()) k_step_pair(const S* __restrict__ src, S* __restrict__ dst,
                                                                           const float* __restrict__ Ff, PR<float> p,
